@@ -31,7 +31,10 @@ struct PassArgs {
     typename Cx<R>::V *adj;    // nullable: receives P psi in the store
     const uint8_t *cost;
     double *partials;          // [batch][gridDim.x][2] when reduce
-    int n, row, lo, m;
+    const int *slots;          // SYM_CHECK, nullable: [batch][nslots] verdicts of flip_check_kernel
+    int nslots;
+    int expand;                // SYM_CHECK: the pass also writes the other half of the state
+    int n, row, lo, m;         // n: index bits; with SYM_CHECK n, lo, tiles are the full state's
     uint32_t active;           // tile bits to butterfly
     int reduce;
     int ua1, ua2;              // butterfly forms of the two layers (fused: l, l+1)
@@ -43,6 +46,57 @@ template <typename R, int NT>
 struct PhaseTab {
     typename Cx<R>::V t[NT];
 };
+
+// Which assignments a pass works on (the state's global flip: psi(x) =
+// psi(not x) when C(x) = C(not x) for every x).  A compile-time choice: one
+// kernel that took either cost the halved state's high passes 1.2% (24 x n = 24,
+// p = 10: 6.16 -> 6.24 ms), their plan then being a runtime value.
+enum SymMode {
+    SYM_HALF = 0,   // the caller's halved state and table (QAOA_Z2_HALF)
+    SYM_CHECK = 1,  // a full table: the 2^(n-1) amplitudes with bit n-1 clear when
+                    // its slots say it is flip-symmetric; else (or with no slots) all
+};
+
+// Is the table of instance blockIdx.y flip-symmetric, C(x) = C(2^n - 1 - x)?
+// Every NAE table is (Sec. 2.2); a caller's own table need not be.  The slot of
+// each block is nonzero when one of its 16-byte words of the lower half
+// differs from the reversed word of the upper half.
+//
+// Bound by the read of the table (2^30 bytes in 0.18 ms, 6.0 TB/s), against the
+// 17 B per amplitude and layer that the halved passes then save on half of the
+// amplitudes; at small n by its launch.
+constexpr int CHECK_PT = 512;
+__global__ void __launch_bounds__(CHECK_PT) flip_check_kernel(const uint8_t *cost, int n, int *slots) {
+    const uint4 *c = reinterpret_cast<const uint4 *>(cost + ((size_t)blockIdx.y << n));
+    const uint32_t W = 1u << (n - 4), H = W / 2, step = gridDim.x * CHECK_PT;
+    uint32_t bad = 0;
+    auto rev = [](uint32_t v) { return __byte_perm(v, 0, 0x0123); };
+    auto differs = [&](const uint4 &a, const uint4 &b) {
+        return (a.x ^ rev(b.w)) | (a.y ^ rev(b.z)) | (a.z ^ rev(b.y)) | (a.w ^ rev(b.x));
+    };
+    uint32_t w = blockIdx.x * CHECK_PT + threadIdx.x;
+    for (; w < H && H - w > 3 * step; w += 4 * step) {  // four words of each half in flight
+        uint4 a[4], b[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = __ldg(c + w + j * step);
+            b[j] = __ldg(c + (W - 1 - w - j * step));
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) bad |= differs(a[j], b[j]);
+    }
+    for (; w < H; w += step) bad |= differs(__ldg(c + w), __ldg(c + (W - 1 - w)));
+    const int any = __syncthreads_or(bad != 0);
+    if (threadIdx.x == 0) slots[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = any;
+}
+
+// Blocks per instance of the check (its slots): 16 KiB of table each, at most
+// two per SM over the batch (every pass CTA reads its instance's slots).
+int flip_slots(int n, int batch, int sms) {
+    const uint64_t need = n > 14 ? 1ull << (n - 14) : 1ull;
+    const uint64_t cap = std::max(1, 2 * sms / batch);
+    return (int)std::min(need, cap);
+}
 
 // Pass modes (MODE_* in the internal header): INIT generates layer 0's state
 // from the phase table, PHASE multiplies by a layer's phase at load, PLAIN only
@@ -115,7 +169,9 @@ __host__ __device__ __forceinline__ constexpr uint32_t land(uint32_t u) {
 // first element; register r adds the state offset of tile element r << LO,
 // i.e. its row part plus its group part times gstride = 2^lo (ROW: the
 // tile's row bits).  In the halved state's mirror half (low pass) the offsets
-// run downwards.  Indices inside one instance fit in 32 bits (n <= 32).
+// run downwards.  mp (nullable): where the first element's complement goes in
+// the other half of a full state; the others run the opposite way.  Indices
+// inside one instance fit in 32 bits (n <= 32).
 // sc: the tile's cost bytes in shared memory, indexed by tile element (by
 // landing position when Z2).
 // |v|^2 and a zero amplitude for each arithmetic (double-float: in FP64).
@@ -142,8 +198,8 @@ constexpr bool is_df() {
 
 template <typename R, int LO, int ROW, bool Z2, bool RED, bool PADC>
 __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename Cx<R>::V *sp, const uint8_t *sc,
-                                           typename Cx<R>::V *sa, uint32_t gstride, bool mirror, bool reduce,
-                                           double acc[2]) {
+                                           typename Cx<R>::V *sa, typename Cx<R>::V *mp, uint32_t gstride, bool mirror,
+                                           bool reduce, double acc[2]) {
     using V = typename Cx<R>::V;
     using P = decltype(amp_prob(v[0]));  // probability accumulation type
     constexpr int NR = Cx<R>::NR;
@@ -160,7 +216,9 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const float4 w = *reinterpret_cast<const float4 *>(&v[r]);
-            sd[off(r)] = make_double2((double)w.x + (double)w.y, (double)w.z + (double)w.w);
+            const double2 d = make_double2((double)w.x + (double)w.y, (double)w.z + (double)w.w);
+            sd[off(r)] = d;
+            if (mp) reinterpret_cast<double2 *>(mp)[-off(r)] = d;
         }
     } else if constexpr (is_df<R>()) {  // pairs renormalised between passes
 #pragma unroll
@@ -168,6 +226,10 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
     } else {
 #pragma unroll
         for (int r = 0; r < NR; ++r) sp[off(r)] = v[r];
+        if (RED && mp) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) mp[-off(r)] = v[r];
+        }
     }
     if (RED && reduce) {
         // The thread's NR probabilities are summed pairwise in P (FP32 for
@@ -244,8 +306,8 @@ __host__ __device__ constexpr bool early_landing() {
 // (and cost) buffers, one CTA per SM; tile i + 2's copies are issued when tile
 // i starts, so two tiles are always in flight while one is computed (a
 // cp.async commit-group pipeline: wait_group 2 completes the oldest).
-template <typename R, bool LOW, int MODE, bool UA1, bool UA2, bool Z2, bool RED, int HROW, bool FULL, int NB>
-__device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename Cx<R>::V *stab,
+template <typename R, bool LOW, int MODE, bool UA1, bool UA2, bool Z2, bool RED, int HROW, bool FULL, int NB, int SYM>
+__device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half, const typename Cx<R>::V *stab,
                                            typename Cx<R>::V *tiles_buf, uint8_t *scs, typename Cx<R>::V *ebuf) {
     using G = Cx<R>;
     using V = typename G::V;
@@ -257,6 +319,11 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename 
     V *st = a.state + (inst << a.n);
     V *adj = a.adj ? a.adj + (inst << a.n) : nullptr;
     const uint8_t *cs = a.cost + (inst << a.n);
+    // The halved plan has the full plan's groups one bit lower (the low pass
+    // covers T - 1 bits and the mirror), so the two share their launches.
+    const bool shift = SYM == SYM_CHECK && half;
+    const int nb = shift ? a.n - 1 : a.n;
+    const int lo = LOW ? T : (shift ? a.lo - 1 : a.lo);
     // Only the evolution's last pass reduces (a plain pass, or the initial one
     // when p = 0); RED compiles that path in.
     const bool red = RED && a.reduce;
@@ -271,21 +338,22 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename 
     // Stores go straight from registers: thread pointer + the register's offset.
     static_assert(!Z2 || (LOW && MODE != MODE_FUSED), "the halved state changes the low pass only");
     // State indices of one instance fit in 32 bits (n <= 32).
-    const uint32_t ld_t = elem_offset32(tile_elem<G, LD>(tid, 0), row, a.lo);
-    const uint32_t st_t = elem_offset32(tile_elem<G, LC>(tid, 0), row, a.lo);
-    const uint32_t gstride = LOW ? 0u : (1u << a.lo);
+    const uint32_t ld_t = elem_offset32(tile_elem<G, LD>(tid, 0), row, lo);
+    const uint32_t st_t = elem_offset32(tile_elem<G, LC>(tid, 0), row, lo);
+    const uint32_t gstride = LOW ? 0u : (1u << lo);
     // halved state: the mirror of element x of the stored half is M - x
-    const uint32_t M = (uint32_t)((1ull << a.n) - 1);
+    const uint32_t M = (uint32_t)((1ull << nb) - 1);
+    const bool expand = RED && shift && a.expand;  // element x also goes to its complement 2 M + 1 - x
     constexpr uint32_t H = 1u << (T - 1);
     const uint32_t z_u0 = tile_elem<G, LC>(tid, 0);  // its bit T - 1 is a thread bit in every store mapping
     const bool z_mir = Z2 && (z_u0 >> (T - 1));
-    auto base_of = [&](uint32_t tt) { return Z2 ? (tt << (T - 1)) : tile_base32(tt, row, a.lo, T); };
+    auto base_of = [&](uint32_t tt) { return Z2 ? (tt << (T - 1)) : tile_base32(tt, row, lo, T); };
     auto issue = [&](uint32_t tt, V *tb, uint8_t *scb) {
         const uint32_t bb = base_of(tt);
         if (Z2)
             issue_tile_z2<R>(st, cs, bb, M - bb - (H - 1), need_s, need_c, tb, scb);
         else
-            issue_tile<Cx<R>, !LOW>(st, cs, bb, row, a.lo, need_s, need_c, tb, scb);
+            issue_tile<Cx<R>, !LOW>(st, cs, bb, row, lo, need_s, need_c, tb, scb);
     };
     auto tbuf = [&](int b) { return tiles_buf + (size_t)b * G::TILE_ELEMS; };
     auto cbuf = [&](int b) { return scs + (size_t)b * G::CS_BYTES; };
@@ -296,14 +364,14 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename 
                   "the early part must be whole registers and whole copy chunks");
     auto issue_early = [&](uint32_t tt, uint8_t *scb) {  // elements below EARLY_ELEMS and the cost bytes
         if constexpr (EARLY)
-            issue_tile<Cx<R>, true, 0, JE>(st, cs, base_of(tt), row, a.lo, true, true, ebuf, scb);
+            issue_tile<Cx<R>, true, 0, JE>(st, cs, base_of(tt), row, lo, true, true, ebuf, scb);
     };
     auto issue_late = [&](uint32_t tt, V *tb) {  // the other elements, into the tile buffer
         if constexpr (EARLY)
-            issue_tile<Cx<R>, true, JE, -1>(st, cs, base_of(tt), row, a.lo, true, false, tb, nullptr);
+            issue_tile<Cx<R>, true, JE, -1>(st, cs, base_of(tt), row, lo, true, false, tb, nullptr);
     };
     double acc[2] = {0.0, 0.0};  // p_succ, norm
-    const uint32_t tiles = (uint32_t)a.tiles;
+    const uint32_t tiles = (uint32_t)(shift ? a.tiles / 2 : a.tiles);
     // High passes that read both the state and the cost bytes take tiles in
     // groups of GT = 64 B / (cost bytes per row): tiles GT q .. GT q + GT - 1,
     // q = blockIdx.x + k gridDim.x.  Their rows are neighbours in memory, so the
@@ -392,16 +460,21 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename 
 #pragma unroll
             for (int r = 0; r < NR; ++r) v[r] = cmul(v[r], stab[sc[cb + G::cidx((uint32_t)r << LC)]]);
             rounds_down<G, LOW, UA2>(v, tile, active, a.A2, a.B2, prefetch);
-            store_tile<R, LD, row, false, false, !LOW>(v, st + (base + ld_t), sc, nullptr, gstride, false, false, acc);
+            store_tile<R, LD, row, false, false, !LOW>(v, st + (base + ld_t), sc, nullptr, nullptr, gstride, false, false,
+                                                       acc);
         } else {
             rounds_up<G, LOW, UA1>(v, tile, active, a.A1, a.B1, prefetch);
             if (Z2) {  // the mirror half stores in descending order
                 const uint32_t ul0 = z_u0 & (H - 1);
-                V *sp = z_mir ? st + (M - base - ul0) : st + (base + ul0);
-                store_tile<R, LC, row, true, RED, false>(v, sp, sc, nullptr, gstride, z_mir, red, acc);
+                const uint32_t x0 = z_mir ? M - base - ul0 : base + ul0;
+                store_tile<R, LC, row, true, RED, false>(v, st + x0, sc, adj ? adj + x0 : nullptr,
+                                                         expand ? st + (2ull * M + 1 - x0) : nullptr, gstride, z_mir,
+                                                         red, acc);
             } else {
-                store_tile<R, LC, row, false, RED, !LOW>(v, st + (base + st_t), sc, adj ? adj + (base + st_t) : nullptr,
-                                                   gstride, false, red, acc);
+                const uint32_t x0 = base + st_t;
+                store_tile<R, LC, row, false, RED, !LOW>(v, st + x0, sc, adj ? adj + x0 : nullptr,
+                                                         expand ? st + (2ull * M + 1 - x0) : nullptr, gstride, false,
+                                                         red, acc);
             }
         }
     }
@@ -409,10 +482,20 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const typename 
         block_sum<2, G::PT>(acc);
         if (threadIdx.x == 0) {
             double *out = a.partials + 2 * (inst * gridDim.x + blockIdx.x);
-            out[0] = acc[0];
-            out[1] = acc[1];
+            // a checked table: each amplitude stands for its complement too
+            // (the caller of a halved state doubles its results itself)
+            const double f = shift ? 2.0 : 1.0;
+            out[0] = f * acc[0];
+            out[1] = f * acc[1];
         }
     }
+}
+
+// Whether every slot of instance blockIdx.y is clear (all threads take part).
+__device__ __forceinline__ bool flip_symmetric(const int *slots, int nslots) {
+    int bad = 0;
+    for (int i = threadIdx.x; i < nslots; i += blockDim.x) bad |= slots[(size_t)blockIdx.y * nslots + i];
+    return !__syncthreads_or(bad);
 }
 
 // Shared-memory phase table length: at least 256 entries (any uint8 cost
@@ -427,12 +510,20 @@ __host__ __device__ __forceinline__ int table_entries(int m) {
 // the phase table.  Cost bytes are padded in high passes.
 // UA1 / UA2: butterfly forms (A = 1 or B = 1) of the pass's one or two layers,
 // chosen on the host per layer.
-template <typename R, bool LOW, int MODE, bool UA1, bool UA2, int NT, bool Z2 = false, bool RED = false,
-          int HROW = HIGH_ROW, bool FULL = true, int NB = 1>
+//
+// A full table whose slots say C(x) = C(not x) is evolved on the half of the
+// assignments with bit n-1 clear, in place in the lower half of the state
+// buffer, and the last pass writes the other half (expand).  The high passes
+// differ only in runtime values; the low pass takes the mirrored tile.  Half
+// the bytes and half the arithmetic per pass, the check and one half's writes
+// more per evolution: n = 30, p = 10 with its table 58.2 -> 30.9 ms (complex64,
+// HBM-bound), n = 26 74.4 -> 37.3 ms (FP64, pipe-bound), n = 27 43.7 -> 21.2 ms
+// (double-float, FP32 issue), n = 21, p = 7 186 -> 178 us (launches).
+template <typename R, int SYM, bool LOW, int MODE, bool UA1, bool UA2, int NT, bool RED = false, int HROW = HIGH_ROW,
+          bool FULL = true, int NB = 1>
 __global__ void __launch_bounds__(Cx<R>::PT, NB == 3 ? 1 : 2) pass_kernel(const __grid_constant__ PassArgs<R> a,
                                                                           const __grid_constant__ PhaseTab<R, NT> tab) {
     using V = typename Cx<R>::V;
-    constexpr int T = Cx<R>::T;
     constexpr int NCB = NB == 3 ? 3 : 2;  // cost buffers
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *tile = reinterpret_cast<V *>(smem_raw);
@@ -444,7 +535,16 @@ __global__ void __launch_bounds__(Cx<R>::PT, NB == 3 ? 1 : 2) pass_kernel(const 
         for (int i = threadIdx.x; i < 256 || i <= a.m; i += Cx<R>::PT) stab[i] = i <= a.m ? tab.t[i] : zero_amp<V>();
         __syncthreads();
     }
-    pass_tiles<R, LOW, MODE, UA1, UA2, Z2, RED, HROW, FULL, NB>(a, stab, tile, scs, ebuf);
+    bool half = SYM == SYM_HALF;
+    if constexpr (SYM == SYM_CHECK) {
+        if (a.slots) half = flip_symmetric(a.slots, a.nslots);
+    }
+    if constexpr (!LOW)
+        pass_tiles<R, LOW, MODE, UA1, UA2, false, RED, HROW, FULL, NB, SYM>(a, half, stab, tile, scs, ebuf);
+    else if (half)
+        pass_tiles<R, LOW, MODE, UA1, UA2, true, RED, HROW, FULL, NB, SYM>(a, true, stab, tile, scs, ebuf);
+    else
+        pass_tiles<R, LOW, MODE, UA1, UA2, false, RED, HROW, FULL, NB, SYM>(a, false, stab, tile, scs, ebuf);
 }
 
 // Fixed-order reduction of per-block partials: out[b][k] = sum_j part[b][j][k].
@@ -677,21 +777,21 @@ using KPtr = const void *;
 
 // The kernels of one kind of high pass: rows of HROW bits; FULL: every group
 // bit is butterflied.  [ua1] for init / plain, [ua1][ua2] for fused.
-template <typename R, int HROW, bool FULL>
+template <typename R, int SYM, int HROW, bool FULL>
 struct HighSet {
     using Full = PhaseTab<R, MAX_TABLE>;
     using None = PhaseTab<R, 1>;
-    void (*init[2])(PassArgs<R>, Full) = {pass_kernel<R, false, MODE_INIT, false, false, MAX_TABLE, false, false, HROW, FULL>,
-                                          pass_kernel<R, false, MODE_INIT, true, false, MAX_TABLE, false, false, HROW, FULL>};
-    void (*plain[2])(PassArgs<R>, None) = {pass_kernel<R, false, MODE_PLAIN, false, false, 1, false, false, HROW, FULL>,
-                                           pass_kernel<R, false, MODE_PLAIN, true, false, 1, false, false, HROW, FULL>};
-    void (*plain_red[2])(PassArgs<R>, None) = {pass_kernel<R, false, MODE_PLAIN, false, false, 1, false, true, HROW, FULL>,
-                                               pass_kernel<R, false, MODE_PLAIN, true, false, 1, false, true, HROW, FULL>};
+    void (*init[2])(PassArgs<R>, Full) = {pass_kernel<R, SYM, false, MODE_INIT, false, false, MAX_TABLE, false, HROW, FULL>,
+                                          pass_kernel<R, SYM, false, MODE_INIT, true, false, MAX_TABLE, false, HROW, FULL>};
+    void (*plain[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, false, MODE_PLAIN, false, false, 1, false, HROW, FULL>,
+                                           pass_kernel<R, SYM, false, MODE_PLAIN, true, false, 1, false, HROW, FULL>};
+    void (*plain_red[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, false, MODE_PLAIN, false, false, 1, true, HROW, FULL>,
+                                               pass_kernel<R, SYM, false, MODE_PLAIN, true, false, 1, true, HROW, FULL>};
     void (*fused[2][2])(PassArgs<R>, Full) = {
-        {pass_kernel<R, false, MODE_FUSED, false, false, MAX_TABLE, false, false, HROW, FULL>,
-         pass_kernel<R, false, MODE_FUSED, false, true, MAX_TABLE, false, false, HROW, FULL>},
-        {pass_kernel<R, false, MODE_FUSED, true, false, MAX_TABLE, false, false, HROW, FULL>,
-         pass_kernel<R, false, MODE_FUSED, true, true, MAX_TABLE, false, false, HROW, FULL>}};
+        {pass_kernel<R, SYM, false, MODE_FUSED, false, false, MAX_TABLE, false, HROW, FULL>,
+         pass_kernel<R, SYM, false, MODE_FUSED, false, true, MAX_TABLE, false, HROW, FULL>},
+        {pass_kernel<R, SYM, false, MODE_FUSED, true, false, MAX_TABLE, false, HROW, FULL>,
+         pass_kernel<R, SYM, false, MODE_FUSED, true, true, MAX_TABLE, false, HROW, FULL>}};
     void all(std::vector<KPtr> &ks) const {
         for (int i = 0; i < 2; ++i) {
             ks.push_back((KPtr)init[i]);
@@ -702,22 +802,21 @@ struct HighSet {
     }
 };
 
-// The kernels of the low pass (Z2: the halved state's mirror variant; NB:
-// tile buffers per CTA); all butterfly every tile bit, except init0 (p = 0:
-// the initial state alone).
-template <typename R, bool Z2, int NB = 1>
+// The kernels of the low pass (NB: tile buffers per CTA); all butterfly every
+// tile bit, except init0 (p = 0: the initial state alone).
+template <typename R, int SYM, int NB = 1>
 struct LowSet {
     using Full = PhaseTab<R, MAX_TABLE>;
     using None = PhaseTab<R, 1>;
-    void (*init[2])(PassArgs<R>, Full) = {pass_kernel<R, true, MODE_INIT, false, false, MAX_TABLE, Z2, true, HIGH_ROW, true, NB>,
-                                          pass_kernel<R, true, MODE_INIT, true, false, MAX_TABLE, Z2, true, HIGH_ROW, true, NB>};
-    void (*init0)(PassArgs<R>, Full) = pass_kernel<R, true, MODE_INIT, true, false, MAX_TABLE, Z2, true, HIGH_ROW, false, NB>;
-    void (*phase[2])(PassArgs<R>, Full) = {pass_kernel<R, true, MODE_PHASE, false, false, MAX_TABLE, Z2, false, HIGH_ROW, true, NB>,
-                                           pass_kernel<R, true, MODE_PHASE, true, false, MAX_TABLE, Z2, false, HIGH_ROW, true, NB>};
-    void (*plain[2])(PassArgs<R>, None) = {pass_kernel<R, true, MODE_PLAIN, false, false, 1, Z2, false, HIGH_ROW, true, NB>,
-                                           pass_kernel<R, true, MODE_PLAIN, true, false, 1, Z2, false, HIGH_ROW, true, NB>};
-    void (*plain_red[2])(PassArgs<R>, None) = {pass_kernel<R, true, MODE_PLAIN, false, false, 1, Z2, true, HIGH_ROW, true, NB>,
-                                               pass_kernel<R, true, MODE_PLAIN, true, false, 1, Z2, true, HIGH_ROW, true, NB>};
+    void (*init[2])(PassArgs<R>, Full) = {pass_kernel<R, SYM, true, MODE_INIT, false, false, MAX_TABLE, true, HIGH_ROW, true, NB>,
+                                          pass_kernel<R, SYM, true, MODE_INIT, true, false, MAX_TABLE, true, HIGH_ROW, true, NB>};
+    void (*init0)(PassArgs<R>, Full) = pass_kernel<R, SYM, true, MODE_INIT, true, false, MAX_TABLE, true, HIGH_ROW, false, NB>;
+    void (*phase[2])(PassArgs<R>, Full) = {pass_kernel<R, SYM, true, MODE_PHASE, false, false, MAX_TABLE, false, HIGH_ROW, true, NB>,
+                                           pass_kernel<R, SYM, true, MODE_PHASE, true, false, MAX_TABLE, false, HIGH_ROW, true, NB>};
+    void (*plain[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, true, MODE_PLAIN, false, false, 1, false, HIGH_ROW, true, NB>,
+                                           pass_kernel<R, SYM, true, MODE_PLAIN, true, false, 1, false, HIGH_ROW, true, NB>};
+    void (*plain_red[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, true, MODE_PLAIN, false, false, 1, true, HIGH_ROW, true, NB>,
+                                               pass_kernel<R, SYM, true, MODE_PLAIN, true, false, 1, true, HIGH_ROW, true, NB>};
     void all(std::vector<KPtr> &ks) const {
         ks.push_back((KPtr)init0);
         for (int i = 0; i < 2; ++i) {
@@ -729,39 +828,35 @@ struct LowSet {
     }
 };
 
-// Stand-in for the halved-state kernels where an arithmetic has none
-// (double-float evolutions take the full state only).
+// Stand-in for the three-buffer kernels where an arithmetic has none.
 template <typename R>
 struct NoLowSet {
     void all(std::vector<KPtr> &) const {}
 };
 
-template <typename R>
+template <typename R, int SYM>
 struct PassKernels {
     using Full = PhaseTab<R, MAX_TABLE>;
     using None = PhaseTab<R, 1>;
     // high passes with rows of WROW bits (complex64: 32 amplitudes, 256 B);
     // complex128 has no wide rows and those are the narrow kernels again
     static constexpr int WROW = sizeof(R) == 4 ? HIGH_ROW + 1 : HIGH_ROW;
-    LowSet<R, false> low;
-    typename std::conditional<is_df<R>(), NoLowSet<R>, LowSet<R, true>>::type low_z2;
+    LowSet<R, SYM> low;
     // One CTA per SM, three tile buffers: the complex64 low passes of a single
     // instance (full and halved state).  (Measured in same-box A/Bs: the
     // strided high passes, the double-float and complex128 low passes and
     // batched low passes all run slower with one CTA per SM.)
     static constexpr bool NB3 = std::is_same<R, float>::value;
-    typename std::conditional<NB3, LowSet<R, false, 3>, NoLowSet<R>>::type low3;
-    typename std::conditional<NB3, LowSet<R, true, 3>, NoLowSet<R>>::type low_z2_3;
-    HighSet<R, HIGH_ROW, true> high;     // [wide][full] below
-    HighSet<R, HIGH_ROW, false> high_part;
-    HighSet<R, WROW, true> wide;
-    HighSet<R, WROW, false> wide_part;
+    typename std::conditional<NB3, LowSet<R, SYM, 3>, NoLowSet<R>>::type low3;
+    HighSet<R, SYM, HIGH_ROW, true> high;     // [wide][full] below
+    HighSet<R, SYM, HIGH_ROW, false> high_part;
+    HighSet<R, SYM, WROW, true> wide;
+    HighSet<R, SYM, WROW, false> wide_part;
     bool nb3_ok = false;  // the three-buffer kernels' shared memory fits the device
     cudaError_t init(size_t smem_optin) {
         const int big = (int)pass_smem<R>(true, MAX_TABLE - 1, 1, std::is_same<R, float>::value);
         std::vector<KPtr> ks;
         low.all(ks);
-        low_z2.all(ks);
         high.all(ks);
         high_part.all(ks);
         wide.all(ks);
@@ -775,7 +870,6 @@ struct PassKernels {
         if (nb3_ok) {
             std::vector<KPtr> k3;
             low3.all(k3);
-            low_z2_3.all(k3);
             for (KPtr k : k3) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big3);
                 if (e != cudaSuccess) return e;
@@ -785,10 +879,10 @@ struct PassKernels {
     }
 };
 
-template <typename R>
-static int pass_kernels(PassKernels<R> **out) {
+template <typename R, int SYM>
+static int pass_kernels(PassKernels<R, SYM> **out) {
     static std::mutex mu;
-    static PassKernels<R> pk;
+    static PassKernels<R, SYM> pk;
     static int state[MAX_DEVICES] = {};  // per device: 0 = not yet, 1 = ok
     const int dev = current_device_slot();
     if (dev < 0) return QAOA_ECUDA;
@@ -856,7 +950,7 @@ static float4 amp_from(float4 *, double re, double im) {
 }
 
 template <typename R>
-static void fill_table(typename PassKernels<R>::Full *tab, const EvolveReq &r, int l, int sign) {
+static void fill_table(PhaseTab<R, MAX_TABLE> *tab, const EvolveReq &r, int l, int sign) {
     std::vector<double> re(r.m + 1), im(r.m + 1);
     const LayerCoef k = r.p > 0 ? layer_coef(r.beta[l], sign, arith_of(r.dtype, r.flags)) : LayerCoef{1.0, 1.0, 0.0, true};
     double scale = std::pow(k.sigma, r.n);
@@ -865,24 +959,33 @@ static void fill_table(typename PassKernels<R>::Full *tab, const EvolveReq &r, i
     for (int c = 0; c <= r.m; ++c) tab->t[c] = amp_from(&tab->t[c], re[c], im[c]);
 }
 
-template <typename R>
+template <typename R, int SYM>
 static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStream_t stream) {
     using V = typename Cx<R>::V;
-    PassKernels<R> *pk = nullptr;
-    int rc = pass_kernels<R>(&pk);
+    using Kernels = PassKernels<R, SYM>;
+    Kernels *pk = nullptr;
+    int rc = pass_kernels<R, SYM>(&pk);
     if (rc) return rc;
-    const bool z2 = (r.flags & QAOA_Z2_HALF) != 0;
+    // With SYM_CHECK the kernels take the full plan; the halved plan's groups are
+    // its groups one bit lower, and the kernels shift them.
     Plan pl;
-    rc = make_plan(r.n, r.dtype, &pl, z2);
+    rc = make_plan(r.n, r.dtype, &pl, SYM == SYM_HALF);
     if (rc) return rc;
     constexpr int T = Cx<R>::T;
+    const bool check = SYM == SYM_CHECK && r.slots && r.p > 0;
+    if (check) {
+        profile_before(K_FLIP_CHECK, stream);
+        flip_check_kernel<<<dim3(r.nslots, r.batch), CHECK_PT, 0, stream>>>(r.cost, r.n, r.slots);
+        rc = profile_after(K_FLIP_CHECK, stream);
+        if (rc) return rc;
+    }
     const int sign = (r.flags & QAOA_MIXER_RX2B) ? -1 : 1;
     const int arith = arith_of(r.dtype, r.flags);
     const bool want = r.d_result != nullptr;
     // The phase table is large: keep it off the stack.
-    std::vector<char> tbuf(sizeof(typename PassKernels<R>::Full));
-    auto *tab = reinterpret_cast<typename PassKernels<R>::Full *>(tbuf.data());
-    typename PassKernels<R>::None none{};
+    std::vector<char> tbuf(sizeof(typename Kernels::Full));
+    auto *tab = reinterpret_cast<typename Kernels::Full *>(tbuf.data());
+    typename Kernels::None none{};
     const std::vector<Launch> seq = make_schedule(pl.n_passes, r.p);
     const dim3 block(Cx<R>::PT), grid(gx, r.batch);
     // The complex64 low passes of a single instance take the three-buffer
@@ -890,8 +993,8 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
     // per SM (never wider than gx, the partials buffer's width).
     DeviceInfo di;
     if (device_info(&di)) return QAOA_ECUDA;
-    const bool use3 = PassKernels<R>::NB3 && pk->nb3_ok && r.batch == 1;
-    const uint64_t tiles_one = 1ull << (pl.state_bits - T);
+    const bool use3 = Kernels::NB3 && pk->nb3_ok && r.batch == 1;
+    const uint64_t tiles_one = 1ull << (pl.state_bits - (check ? 1 : 0) - T);
     const int gx3 = std::min(balanced_grid_x(di.sms, r.batch, tiles_one), gx);
     const dim3 grid3(gx3, r.batch);
     int last_gx = gx;  // grid width of the pass that writes the p_succ partials
@@ -903,14 +1006,16 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
         a.state = reinterpret_cast<V *>(r.state);
         a.cost = r.cost;
         a.partials = d_partials;
-        a.n = pl.state_bits;  // index bits of the stored state (and of the cost table)
+        a.slots = check ? r.slots : nullptr;
+        a.nslots = r.nslots;
+        a.n = pl.state_bits;  // also the stride of the instances
         a.m = r.m;
         if (low) {  // the whole tile is one contiguous row
             a.row = T;
             a.lo = T;
             a.active = r.p > 0 ? ((1u << T) - 1u) : 0u;
         } else {
-            if (ps.row != HIGH_ROW && ps.row != PassKernels<R>::WROW)
+            if (ps.row != HIGH_ROW && ps.row != Kernels::WROW)
                 return set_error(QAOA_ECUDA, "plan: high pass rows of %d bits", ps.row);
             a.row = ps.row;
             a.lo = ps.lo;
@@ -918,7 +1023,10 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
         }
         const bool last = i + 1 == seq.size();
         // a double-float evolution's last pass always reduces: it writes FP64 out
-        a.reduce = (last && (want || r.adj || is_df<R>())) ? 1 : 0;
+        // as does one on a checked table, where the last pass writes the other half
+        // (not for the gradient, whose backward sweep starts from the halves)
+        a.expand = last && check && !r.adj ? 1 : 0;
+        a.reduce = (last && (want || r.adj || a.expand || is_df<R>())) ? 1 : 0;
         if (a.reduce && !(L.mode == MODE_PLAIN || (L.mode == MODE_INIT && low)))
             return set_error(QAOA_ECUDA, "schedule: the last pass has mode %d", L.mode);
         a.adj = (last && r.adj) ? reinterpret_cast<V *>(r.adj) : nullptr;
@@ -957,18 +1065,9 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
                 return QAOA_OK;
             };
             int lrc = QAOA_OK;
-            if constexpr (PassKernels<R>::NB3) {
+            if constexpr (Kernels::NB3) {
                 const size_t p3 = pass_smem<R>(true, r.m, 3), q3 = pass_smem<R>(false, 0, 3);
-                if (use3)
-                    lrc = z2 ? launch_low(pk->low_z2_3, grid3, p3, q3) : launch_low(pk->low3, grid3, p3, q3);
-                else
-                    lrc = z2 ? launch_low(pk->low_z2, grid, smem_phase, smem_plain)
-                             : launch_low(pk->low, grid, smem_phase, smem_plain);
-            } else if (z2) {
-                if constexpr (is_df<R>())
-                    lrc = set_error(QAOA_EINVAL, "double-float takes the full state");
-                else
-                    lrc = launch_low(pk->low_z2, grid, smem_phase, smem_plain);
+                lrc = use3 ? launch_low(pk->low3, grid3, p3, q3) : launch_low(pk->low, grid, smem_phase, smem_plain);
             } else {
                 lrc = launch_low(pk->low, grid, smem_phase, smem_plain);
             }
@@ -976,10 +1075,10 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
         } else {
             // rows of HIGH_ROW or WROW bits; FULL kernels when no bit of the group is a carried one
             const bool wide = ps.row != HIGH_ROW, full = ps.bits == T - ps.row;
-            const HighSet<R, HIGH_ROW, true> &hn = pk->high;
-            const HighSet<R, HIGH_ROW, false> &hp = pk->high_part;
-            const HighSet<R, PassKernels<R>::WROW, true> &wn = pk->wide;
-            const HighSet<R, PassKernels<R>::WROW, false> &wp = pk->wide_part;
+            const HighSet<R, SYM, HIGH_ROW, true> &hn = pk->high;
+            const HighSet<R, SYM, HIGH_ROW, false> &hp = pk->high_part;
+            const HighSet<R, SYM, Kernels::WROW, true> &wn = pk->wide;
+            const HighSet<R, SYM, Kernels::WROW, false> &wp = pk->wide_part;
             if (L.mode == MODE_INIT) {
                 fill_table<R>(tab, r, 0, sign);
                 auto k = wide ? (full ? wn.init[u1] : wp.init[u1]) : (full ? hn.init[u1] : hp.init[u1]);
@@ -1074,9 +1173,14 @@ static int validate_evolve(int batch, int n, const uint8_t *cost, int m, int p, 
 }
 
 int evolve_device_impl(const EvolveReq &r, cudaStream_t stream, double *d_partials, int gx) {
-    if (r.dtype == QAOA_C64) return evolve_passes<float>(r, d_partials, gx, stream);
-    if (r.flags & QAOA_DF64) return evolve_passes<dfloat>(r, d_partials, gx, stream);
-    return evolve_passes<double>(r, d_partials, gx, stream);
+    const bool half = (r.flags & QAOA_Z2_HALF) != 0;
+    auto run = [&](auto tag) {
+        using R = decltype(tag);
+        return half ? evolve_passes<R, SYM_HALF>(r, d_partials, gx, stream)
+                    : evolve_passes<R, SYM_CHECK>(r, d_partials, gx, stream);
+    };
+    if (r.dtype == QAOA_C64) return run(float{});
+    return (r.flags & QAOA_DF64) ? run(dfloat{}) : run(double{});
 }
 
 }  // namespace qaoa
@@ -1121,13 +1225,21 @@ static int evolve_common(int batch, int n, const uint8_t *d_cost, int m, int p, 
         return QAOA_OK;
     }
     if (n <= small_n_limit(dtype)) return set_error(QAOA_ERANGE, "n=%d too small for the pass path", n);
-    const int gx = pass_grid_x(dtype, z2 ? n - 1 : n, batch);
+    // a full table's evolution works on half of the amplitudes when the table is
+    // flip-symmetric (checked on the device, instance by instance)
+    const int gx = pass_grid_x(dtype, p > 0 || z2 ? n - 1 : n, batch);
     if (gx < 0) return QAOA_ECUDA;
     const size_t part = (size_t)batch * gx * 2 * sizeof(double);
     const size_t res = (size_t)batch * 2 * sizeof(double);
-    rc = scratch_for(stream, part + res + 256, res + 64, &sc);
+    if (!z2 && p > 0) {
+        DeviceInfo di;
+        if ((rc = device_info(&di))) return rc;
+        r.nslots = flip_slots(n, batch, di.sms);
+    }
+    rc = scratch_for(stream, part + res + (size_t)batch * r.nslots * sizeof(int) + 256, res + 64, &sc);
     if (rc) return rc;
     double *d_part = reinterpret_cast<double *>(sc->dev);
+    if (r.nslots) r.slots = reinterpret_cast<int *>(reinterpret_cast<char *>(sc->dev) + part + res);
     if (want) r.d_result = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->dev) + part);
     rc = evolve_device_impl(r, stream, d_part, gx);
     if (rc || !want) return rc;

@@ -64,6 +64,7 @@ enum KernelKind {
     K_ADJ_SEED,
     K_SERVE_SMALL,
     K_SAMPLE,
+    K_FLIP_CHECK,
     K_NUM_KINDS
 };
 // Call before / after a launch on `stream`.  `after` checks the launch status.
@@ -189,11 +190,18 @@ struct EvolveReq {
     void *adj;          // nullable: if set, the last pass also writes P psi into it
     const double *gamma, *beta;
     double *d_result;   // nullable: device [batch][2] (p_succ, norm)
+    // Full tables, p > 0: device [batch][nslots] verdicts of the flip-symmetry
+    // check, which the evolution fills first; a symmetric instance then evolves
+    // half of its amplitudes.  Null: every amplitude is evolved.
+    int *slots = nullptr;
+    int nslots = 0;
 };
 // Runs the passes of `r` on `stream`; d_partials holds batch x gx x 2 doubles
 // (gx from pass_grid_x); r.d_result (if set) receives [batch][2].
 int evolve_device_impl(const EvolveReq &r, cudaStream_t stream, double *d_partials, int gx);
 int pass_grid_x(int dtype, int n, int batch);
+// Slots per instance of the flip-symmetry check.
+int flip_slots(int n, int batch, int sms);
 // Grid width per instance for `batch` instances of `tiles` tiles on `slots`
 // resident CTAs (the wave-balanced choice; 1 <= result <= min(slots, tiles)).
 int balanced_grid_x(int slots, int batch, uint64_t tiles);
