@@ -164,9 +164,10 @@ static int finish_slot(qaoa_server *sv, Slot &s) {
 // Launch one large request on slot s (stream ordered, no host sync).
 static int launch_large(qaoa_server *sv, Slot &s, Req &q) {
     const int dtype = sv->o.dtype;
-    // with QAOA_Z2_HALF the request keeps only the half state (global-flip symmetry)
-    const bool z2 = (sv->o.flags & QAOA_Z2_HALF) != 0;
-    const size_t N = (size_t)1 << (z2 ? q.n - 1 : q.n);
+    // The server makes the tables itself, so they are flip-symmetric, and no
+    // state leaves it: with or without QAOA_Z2_HALF a request keeps only the half
+    // table and state (a burst of 48 requests, n = 14..26, p <= 20: 26.4 -> 14.9 ms).
+    const size_t N = (size_t)1 << (q.n - 1);
     int rc;
     naesat_instance inst{q.n, q.m, q.k, q.var.data(), q.neg.data()};
     // staging: [0..2) stats (u64), [2..4) p_succ, norm; from byte 256 the
@@ -177,15 +178,15 @@ static int launch_large(qaoa_server *sv, Slot &s, Req &q) {
     unsigned long long *d_stats = reinterpret_cast<unsigned long long *>(s.d_stage);
     double *d_res = reinterpret_cast<double *>(s.d_stage + 16);
     QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, 16, s.stream));
-    if ((rc = launch_cost_table_one(&inst, (uint8_t *)s.d_cost, d_stats, s.stream, z2, s.d_stage + 256))) return rc;
-    const int gx = pass_grid_x(dtype, z2 ? q.n - 1 : q.n, 1);
+    if ((rc = launch_cost_table_one(&inst, (uint8_t *)s.d_cost, d_stats, s.stream, true, s.d_stage + 256))) return rc;
+    const int gx = pass_grid_x(dtype, q.n - 1, 1);
     if (gx < 0) return QAOA_ECUDA;
     if (s.part_cap < (size_t)gx * 2) {
         if (s.d_part) cudaFree(s.d_part);
         QAOA_CUDA_TRY(cudaMalloc((void **)&s.d_part, (size_t)gx * 2 * sizeof(double)));
         s.part_cap = (size_t)gx * 2;
     }
-    EvolveReq r{1, q.n, table_top(q.m), q.p, dtype, sv->o.flags, (const uint8_t *)s.d_cost, s.d_state, nullptr,
+    EvolveReq r{1, q.n, table_top(q.m), q.p, dtype, sv->o.flags | QAOA_Z2_HALF, (const uint8_t *)s.d_cost, s.d_state, nullptr,
                 q.gamma.data(), q.beta.data(), d_res};
     if ((rc = evolve_device_impl(r, s.stream, s.d_part, gx))) return rc;
     QAOA_CUDA_TRY(cudaMemcpyAsync(s.h_stage, s.d_stage, 32, cudaMemcpyDeviceToHost, s.stream));
@@ -205,8 +206,7 @@ static int launch_group(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<Re
     const int B = (int)batch.size();
     const Req &q0 = *batch[0];
     const int dtype = sv->o.dtype;
-    const bool z2 = (sv->o.flags & QAOA_Z2_HALF) != 0;
-    const int nb = z2 ? q0.n - 1 : q0.n;  // the half table is the first 2^(n-1) entries
+    const int nb = q0.n - 1;  // half tables (the first 2^(n-1) entries) and states, as in launch_large
     const size_t N = (size_t)1 << nb;
     const int m_stride = std::max(q0.m, 1);
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -247,9 +247,9 @@ static int launch_group(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<Re
     QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, (size_t)B * 2 * sizeof(unsigned long long), s.stream));
     if ((rc = launch_cost_table_batch(B, nb, nullptr, nullptr, reinterpret_cast<const ClauseRec *>(d + o_recs),
                                       reinterpret_cast<const int *>(d + o_m), m_stride, (uint8_t *)s.d_cost, d_stats,
-                                      s.stream, !z2)))
+                                      s.stream, false)))
         return rc;
-    EvolveReq r{B, q0.n, table_top(q0.m), q0.p, dtype, sv->o.flags, (const uint8_t *)s.d_cost, s.d_state, nullptr,
+    EvolveReq r{B, q0.n, table_top(q0.m), q0.p, dtype, sv->o.flags | QAOA_Z2_HALF, (const uint8_t *)s.d_cost, s.d_state, nullptr,
                 q0.gamma.data(), q0.beta.data(), d_res};
     if ((rc = evolve_device_impl(r, s.stream, s.d_part, gx))) return rc;
     QAOA_CUDA_TRY(cudaMemcpyAsync(h + o_stats, d + o_stats, total - o_stats, cudaMemcpyDeviceToHost, s.stream));
@@ -356,6 +356,8 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
     return finish_slot(sv, s);
 }
 
+// Bytes a request is charged for: without QAOA_Z2_HALF those of the full table
+// and state, though the unpacked launches allocate half of each.
 static size_t footprint(const qaoa_server *sv, int n, bool packed) {
     const size_t N = (size_t)1 << n;
     if (packed) return N;
@@ -387,7 +389,7 @@ static void retire(qaoa_server *sv, Slot &s) {
             const unsigned long long *st = reinterpret_cast<const unsigned long long *>(s.h_stage + s.res_off);
             const double *res = reinterpret_cast<const double *>(
                 s.h_stage + ((s.res_off + (size_t)B * 16 + 255) & ~(size_t)255));
-            const double f = (sv->o.flags & QAOA_Z2_HALF) ? 2.0 : 1.0;
+            const double f = 2.0;
             r.n_sol = (uint64_t)(f * (double)st[2 * b]);
             r.max_cost = (uint32_t)st[2 * b + 1];
             r.p_succ = f * res[2 * b];
@@ -395,7 +397,7 @@ static void retire(qaoa_server *sv, Slot &s) {
         } else {
             const unsigned long long *st = reinterpret_cast<const unsigned long long *>(s.h_stage);
             const double *res = reinterpret_cast<const double *>(s.h_stage + 16);
-            const double f = (sv->o.flags & QAOA_Z2_HALF) ? 2.0 : 1.0;  // halved state and table
+            const double f = 2.0;  // halved state and table
             r.n_sol = (uint64_t)(f * (double)st[0]);
             r.max_cost = (uint32_t)st[1];
             r.p_succ = f * res[0];
