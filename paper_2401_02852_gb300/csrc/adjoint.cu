@@ -19,6 +19,7 @@
 // computes the same derivative without storing the p intermediate states.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <type_traits>
@@ -38,6 +39,8 @@ struct AdjArgs {
     const uint8_t *cost;
     double *partials;   // layer l's slice: [batch][p][gx][2], base at layer l
     double *partials2;  // A_FUSED: layer l - 1's slice (nullable: no second layer)
+    const int *slots;   // [batch][nslots] verdicts of the flip-symmetry check
+    int nslots;
     int n, row, lo, m, p;
     uint32_t active;
     R c, S;             // inverse butterfly coefficients of layer l
@@ -131,9 +134,16 @@ __device__ __forceinline__ uint32_t reg_off(int r, uint32_t gstride) {
 // the load mapping's register bits, so the pass needs no exchange: the next
 // pair is copied as soon as this one is in registers, and the phase is taken
 // in the load mapping.
-template <typename R, bool LOW, int MODE, int NT, int HROW, int FULL>
-__global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const __grid_constant__ AdjArgs<R> a,
-                                                                        const __grid_constant__ AdjTab<R, NT> tab) {
+//
+// An instance whose table is flip-symmetric has its states in the lower halves
+// of their buffers (the amplitudes with bit n-1 clear), as the forward passes
+// leave them: the groups are then one bit lower, the low pass (Z2) pairs a
+// half-tile with its mirror block, and every sum counts twice.
+// Half the bytes of every pass: 32 x (n = 22, p = 20) complex64 42.2 -> 23.1 ms.
+template <typename R, bool LOW, int MODE, int HROW, int FULL, bool Z2>
+__device__ __forceinline__ void adj_tiles(const AdjArgs<R> &a, const bool half, typename AGeo<R>::V *tp,
+                                          uint8_t *scs, const typename AGeo<R>::V *stab) {
+    static_assert(!Z2 || LOW, "the halved state changes the low pass only");
     static_assert(!LOW || MODE != A_FUSED, "the low pass never fuses");
     static_assert(LOW || MODE != A_PHASE, "a high pass undoes a phase in its fused form");
     constexpr bool PH = MODE != A_PLAIN;  // the pass undoes a phase
@@ -146,36 +156,37 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
     constexpr uint32_t full_mask = ((1u << T) - 1u) & ~(LOW ? 0u : (1u << row) - 1u);
     constexpr bool TOP = !LOW && FULL == 2;
     const uint32_t active = FULL == 1 ? full_mask : a.active;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    V *tp = reinterpret_cast<V *>(smem_raw);
     V *tl = tp + G::TILE_ELEMS;
     // phase passes: two dense cost-byte buffers.  (The forward high passes pad
     // theirs so that the cost loads in mapping 4 take one wavefront instead of
     // two; here the extra per-thread offset made the fused kernels, which hold
     // both states in registers, spill, so the backward passes keep the dense
     // layout and its second wavefront.)
-    uint8_t *scs = reinterpret_cast<uint8_t *>(tl + G::TILE_ELEMS);
-    V *stab = reinterpret_cast<V *>(scs + (PH ? (2 << T) : 0));
-    if (PH) {  // 256 entries at least: any uint8 cost indexes inside the table
-        for (int i = threadIdx.x; i < 256 || i <= a.m; i += PT) {
-            V z;
-            z.x = z.y = 0;
-            stab[i] = i <= a.m ? tab.t[i] : z;
-        }
-    }
     const uint32_t tid = threadIdx.x;
     const size_t inst = blockIdx.y;
     V *psi = a.psi + (inst << a.n);
     V *lam = a.lam + (inst << a.n);
     const uint8_t *cs = a.cost + (inst << a.n);
     constexpr int SM = (MODE == A_FUSED || TOP) ? LD : LC;  // store mapping
-    const uint32_t st_t = elem_offset32(tile_elem<G, SM>(tid, 0), row, a.lo);
-    const uint32_t gstride = LOW ? 0u : (1u << a.lo);
-    const uint32_t tiles = (uint32_t)a.tiles;
+    const int lo = LOW ? T : (half ? a.lo - 1 : a.lo);
+    const uint32_t st_t = elem_offset32(tile_elem<G, SM>(tid, 0), row, lo);
+    const uint32_t gstride = LOW ? 0u : (1u << lo);
+    const uint32_t tiles = (uint32_t)(half ? a.tiles / 2 : a.tiles);
+    // halved state: the mirror of element x of the stored half is M - x
+    const uint32_t M = (uint32_t)((1ull << (a.n - 1)) - 1);
+    constexpr uint32_t H = 1u << (T - 1);
+    const bool z_mir = Z2 && (tile_elem<G, SM>(tid, 0) >> (T - 1));  // a thread bit in the low pass's store mapping
+    auto base_of = [&](uint32_t tt) { return Z2 ? tt << (T - 1) : tile_base32(tt, row, lo, T); };
+    auto pos = [](uint32_t u) { return Z2 ? land<T>(u) : u; };  // landing position of tile element u
     auto issue = [&](uint32_t tt, uint8_t *scb) {
-        const uint32_t bb = tile_base32(tt, row, a.lo, T);
-        issue_tile<G>(psi, cs, bb, row, a.lo, true, PH, tp, scb);
-        issue_tile<G>(lam, cs, bb, row, a.lo, true, false, tl, scb);
+        const uint32_t bb = base_of(tt);
+        if (Z2) {
+            issue_tile_z2<G>(psi, cs, bb, M - bb - (H - 1), true, PH, tp, scb);
+            issue_tile_z2<G>(lam, cs, bb, M - bb - (H - 1), true, false, tl, scb);
+        } else {
+            issue_tile<G>(psi, cs, bb, row, lo, true, PH, tp, scb);
+            issue_tile<G>(lam, cs, bb, row, lo, true, false, tl, scb);
+        }
     };
     double acc[3] = {0.0, 0.0, 0.0};  // mixer term, phase term (layer l), mixer term (layer l - 1)
     uint32_t t = blockIdx.x;
@@ -184,14 +195,14 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
     for (int i = 0; t < tiles; ++i, t += gridDim.x) {
         const int b = i & 1;
         const uint8_t *sc = scs + ((size_t)b << T);
-        const uint32_t base = tile_base32(t, row, a.lo, T);
+        const uint32_t base = base_of(t);
         const uint32_t tn = t + gridDim.x;
         cp_async_wait_all();
         __syncthreads();
         V vp[NR], vl[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {  // dense buffers, consecutive lanes: no conflicts
-            const uint32_t u = tile_elem<G, LD>(tid, r);
+            const uint32_t u = pos(tile_elem<G, LD>(tid, r));
             vp[r] = tp[u];
             vl[r] = tl[u];
         }
@@ -207,7 +218,7 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
             constexpr int MP = decltype(mp)::value;
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-                const int cst = sc[tile_elem<G, MP>(tid, r)];
+                const int cst = sc[pos(tile_elem<G, MP>(tid, r))];
                 gterm += (R)cst * (vl[r].x * vp[r].y - vl[r].y * vp[r].x);
                 const V ph = stab[cst];
                 vp[r] = cmul(vp[r], ph);
@@ -241,15 +252,21 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
             prefetch();
             inv_round<G, LC, LD>(vp, vl, active, a.c, a.S, term);
         }
-        V *pp = psi + (base + st_t);
-        V *pl = lam + (base + st_t);
+        const uint32_t x0 = z_mir ? M - base - (st_t & (H - 1)) : base + st_t;
+        V *pp = psi + x0;
+        V *pl = lam + x0;
         uint32_t gs = gstride;
         asm volatile("" : "+l"(pp), "+l"(pl), "+r"(gs));  // keep the store addresses out of the load phase
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const uint32_t o = reg_off<SM, row>(r, gs);
-            pp[o] = vp[r];
-            pl[o] = vl[r];
+            if (z_mir) {  // the mirror half stores in descending order
+                *(pp - o) = vp[r];
+                *(pl - o) = vl[r];
+            } else {
+                pp[o] = vp[r];
+                pl[o] = vl[r];
+            }
         }
         acc[0] += (double)term;
         acc[1] += (double)gterm;
@@ -258,9 +275,50 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
     block_sum<3>(acc);
     if (threadIdx.x == 0) {
         const size_t slot = 2 * ((inst * a.p) * gridDim.x + blockIdx.x);
-        a.partials[slot] += acc[0];
-        a.partials[slot + 1] += acc[1];
-        if (MODE == A_FUSED && a.partials2) a.partials2[slot] += acc[2];
+        const double f = half ? 2.0 : 1.0;
+        a.partials[slot] += f * acc[0];
+        a.partials[slot + 1] += f * acc[1];
+        if (MODE == A_FUSED && a.partials2) a.partials2[slot] += f * acc[2];
+    }
+}
+
+template <typename R, bool LOW, int MODE, int NT, int HROW, int FULL>
+__global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const __grid_constant__ AdjArgs<R> a,
+                                                                        const __grid_constant__ AdjTab<R, NT> tab) {
+    using G = AGeo<R>;
+    using V = typename G::V;
+    constexpr bool PH = MODE != A_PLAIN;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V *tp = reinterpret_cast<V *>(smem_raw);
+    uint8_t *scs = reinterpret_cast<uint8_t *>(tp + 2 * G::TILE_ELEMS);
+    V *stab = reinterpret_cast<V *>(scs + (PH ? (2 << G::T) : 0));
+    if (PH) {  // 256 entries at least: any uint8 cost indexes inside the table
+        for (int i = threadIdx.x; i < 256 || i <= a.m; i += PT) {
+            V z;
+            z.x = z.y = 0;
+            stab[i] = i <= a.m ? tab.t[i] : z;
+        }
+    }
+    const bool half = flip_symmetric(a.slots, a.nslots);
+    if constexpr (!LOW)
+        adj_tiles<R, LOW, MODE, HROW, FULL, false>(a, half, tp, scs, stab);
+    else if (half)
+        adj_tiles<R, LOW, MODE, HROW, FULL, true>(a, true, tp, scs, stab);
+    else
+        adj_tiles<R, LOW, MODE, HROW, FULL, false>(a, false, tp, scs, stab);
+}
+
+// The other halves of both states of a flip-symmetric instance, once the
+// backward sweep is done: element x goes to its complement N - 1 - x.
+template <typename V>
+__global__ void __launch_bounds__(PT) mirror_kernel(V *psi, V *lam, int n, const int *slots, int nslots) {
+    if (!flip_symmetric(slots, nslots)) return;
+    const size_t N = (size_t)1 << n, off = (size_t)blockIdx.y << n;
+    psi += off;
+    lam += off;
+    for (size_t x = (size_t)blockIdx.x * PT + threadIdx.x; x < N / 2; x += (size_t)gridDim.x * PT) {
+        psi[N - 1 - x] = psi[x];
+        lam[N - 1 - x] = lam[x];
     }
 }
 
@@ -431,16 +489,19 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
     if (rc) return rc;
     const int sign = (flags & QAOA_MIXER_RX2B) ? -1 : 1;
     // forward with the adjoint seed lam_p = P psi_p written by the last pass
-    const int gxf = pass_grid_x(dtype, n, batch);
+    const int gxf = pass_grid_x(dtype, n - 1, batch);
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
     const uint64_t tiles = 1ull << (n - AGeo<R>::T);
-    const int gxa = balanced_grid_x(di.sms * (sizeof(R) == 4 ? 2 : 1), batch, tiles);
+    const int gxa = balanced_grid_x(di.sms * (sizeof(R) == 4 ? 2 : 1), batch, tiles / 2);
     double *d_fpart = d_scr;                                  // batch * gxf * 2
     double *d_fres = d_fpart + (size_t)batch * gxf * 2;       // batch * 2
     double *d_apart = d_fres + (size_t)batch * 2;             // batch * p * gxa * 2
     double *d_ares = d_apart + (size_t)batch * p * gxa * 2;   // batch * p * 2
-    EvolveReq r{batch, n, m, p, dtype, flags, cost, state, adj, gamma, beta, d_fres};
+    // verdicts of the flip-symmetry check, written ahead of the forward passes
+    const int nslots = flip_slots(n, batch, di.sms);
+    int *d_slots = reinterpret_cast<int *>(d_ares + (size_t)batch * p * 2);
+    EvolveReq r{batch, n, m, p, dtype, flags, cost, state, adj, gamma, beta, d_fres, d_slots, nslots};
     if ((rc = evolve_device_impl(r, stream, d_fpart, gxf))) return rc;
     QAOA_CUDA_TRY(cudaMemsetAsync(d_apart, 0, (size_t)batch * p * gxa * 2 * sizeof(double), stream));
     Plan pl;
@@ -459,6 +520,8 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
         a.cost = cost;
         a.partials = d_apart + (size_t)l * gxa * 2;
         a.partials2 = nullptr;
+        a.slots = d_slots;
+        a.nslots = nslots;
         a.n = n;
         a.m = m;
         a.p = p;
@@ -508,6 +571,10 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
         }
         if (rc) return rc;
     }
+    profile_before(K_MIRROR, stream);
+    mirror_kernel<V><<<dim3((unsigned)std::min<uint64_t>(1ull << (n - 9), (uint64_t)di.sms * 8 / batch + 1), batch), PT, 0,
+                       stream>>>(reinterpret_cast<V *>(state), reinterpret_cast<V *>(adj), n, d_slots, nslots);
+    if ((rc = profile_after(K_MIRROR, stream))) return rc;
     if ((rc = launch_reduce(d_apart, batch * p, gxa, 2, d_ares, stream))) return rc;
     QAOA_CUDA_TRY(cudaMemcpyAsync(h_scr, d_fres, (size_t)batch * 2 * sizeof(double), cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaMemcpyAsync(h_scr + 2 * batch, d_ares, (size_t)batch * p * 2 * sizeof(double),
@@ -595,10 +662,10 @@ static int grad_common(int batch, int n, const uint8_t *cost, int m, int p, cons
     }
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
-    const int gxf = pass_grid_x(dtype, n, batch);
+    const int gxf = pass_grid_x(dtype, n - 1, batch);
     const size_t gxa = (size_t)di.sms * 2 + 1;
     const size_t words = (size_t)batch * gxf * 2 + (size_t)batch * 2 + (size_t)batch * p * gxa * 2 +
-                         (size_t)batch * p * 2 + 64;
+                         (size_t)batch * p * 2 + ((size_t)batch * flip_slots(n, batch, di.sms) + 1) / 2 + 64;
     const size_t hwords = (size_t)batch * 2 + (size_t)batch * p * 2 + 16;
     if ((rc = scratch_for(stream, words * sizeof(double), hwords * sizeof(double), &sc))) return rc;
     if (dtype == QAOA_C64)

@@ -156,14 +156,6 @@ __device__ __forceinline__ void rounds_down(typename G::V *v, typename G::V *til
     mask_butterflies<G, UA, P::R0::LO, P::R0::MASK>(v, active, A, B);
 }
 
-// Halved state (low pass): tile element u with bit T-1 set is the mirror
-// 2^(n-1) - 1 - x of the element x = u with that bit clear; its data and cost
-// bytes land in reverse memory order at position 2^T - 1 - (u mod 2^(T-1)).
-template <int T>
-__host__ __device__ __forceinline__ constexpr uint32_t land(uint32_t u) {
-    return (u >> (T - 1)) ? ((1u << T) - 1u - (u & ((1u << (T - 1)) - 1u))) : u;
-}
-
 // Stores the tile from mapping LO, fusing the p_succ / norm partials and the
 // adjoint seed P psi when this is the evolution's last pass.  sp: the thread's
 // first element; register r adds the state offset of tile element r << LO,
@@ -252,41 +244,6 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
     }
 }
 
-// Halved state, low pass: the tile is the half-tile [base, base + H) and its
-// mirror block [mbase, mbase + H), H = 2^(T-1), each copied in memory order
-// (the mirror block lands at positions [H, 2H)).
-template <typename R>
-__device__ __forceinline__ void issue_tile_z2(const typename Cx<R>::V *st, const uint8_t *cs, uint32_t base,
-                                              uint32_t mbase, bool state, bool cost, typename Cx<R>::V *buf,
-                                              uint8_t *sc) {
-    using V = typename Cx<R>::V;
-    constexpr int T = Cx<R>::T;
-    constexpr int EPC = 16 / (int)sizeof(V);
-    constexpr int NT = Cx<R>::PT;
-    constexpr int NCH = (1 << T) / EPC / NT;
-    constexpr int CCH = (1 << T) / 16 / NT;
-    constexpr uint32_t HC = (1u << (T - 1)) / 16;  // cost chunks per half
-    const uint32_t tid = threadIdx.x;
-    if (state) {
-        char *dst = reinterpret_cast<char *>(buf) + 16 * tid;
-        const V *reg = st + base + EPC * tid;
-        const V *mir = st + mbase + EPC * tid;
-#pragma unroll
-        for (int j = 0; j < NCH; ++j) {
-            const V *src = j < NCH / 2 ? reg + (size_t)EPC * NT * j : mir + (size_t)EPC * NT * (j - NCH / 2);
-            cp_async16(dst + (size_t)16 * NT * j, src);
-        }
-    }
-    if (cost) {
-#pragma unroll
-        for (int j = 0; j < CCH; ++j) {
-            const uint32_t q = tid + NT * j;
-            const uint8_t *src = q < HC ? cs + base + 16 * q : cs + mbase + 16 * (q - HC);
-            cp_async16(sc + 16 * q, src);
-        }
-    }
-}
-
 // Early landing (complex64 fused high passes): the next tile's elements
 // u < EARLY_ELEMS and all its cost bytes are copied into buffers of their own
 // right after the current tile's first exchange, i.e. about half a tile of
@@ -351,7 +308,7 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half
     auto issue = [&](uint32_t tt, V *tb, uint8_t *scb) {
         const uint32_t bb = base_of(tt);
         if (Z2)
-            issue_tile_z2<R>(st, cs, bb, M - bb - (H - 1), need_s, need_c, tb, scb);
+            issue_tile_z2<G>(st, cs, bb, M - bb - (H - 1), need_s, need_c, tb, scb);
         else
             issue_tile<Cx<R>, !LOW>(st, cs, bb, row, lo, need_s, need_c, tb, scb);
     };
@@ -489,13 +446,6 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half
             out[1] = f * acc[1];
         }
     }
-}
-
-// Whether every slot of instance blockIdx.y is clear (all threads take part).
-__device__ __forceinline__ bool flip_symmetric(const int *slots, int nslots) {
-    int bad = 0;
-    for (int i = threadIdx.x; i < nslots; i += blockDim.x) bad |= slots[(size_t)blockIdx.y * nslots + i];
-    return !__syncthreads_or(bad);
 }
 
 // Shared-memory phase table length: at least 256 entries (any uint8 cost

@@ -400,6 +400,55 @@ __device__ __forceinline__ void issue_tile(const typename G::V *st, const uint8_
     }
 }
 
+// Halved state (low pass): tile element u with bit T-1 set is the mirror
+// 2^(n-1) - 1 - x of the element x = u with that bit clear; its data and cost
+// bytes land in reverse memory order at position 2^T - 1 - (u mod 2^(T-1)).
+template <int T>
+__host__ __device__ __forceinline__ constexpr uint32_t land(uint32_t u) {
+    return (u >> (T - 1)) ? ((1u << T) - 1u - (u & ((1u << (T - 1)) - 1u))) : u;
+}
+
+// Halved state, low pass: the tile is the half-tile [base, base + H) and its
+// mirror block [mbase, mbase + H), H = 2^(T-1), each copied in memory order
+// (the mirror block lands at positions [H, 2H)).
+template <typename G>
+__device__ __forceinline__ void issue_tile_z2(const typename G::V *st, const uint8_t *cs, uint32_t base,
+                                              uint32_t mbase, bool state, bool cost, typename G::V *buf, uint8_t *sc) {
+    using V = typename G::V;
+    constexpr int T = G::T;
+    constexpr int EPC = 16 / (int)sizeof(V);
+    constexpr int NT = G::PT;
+    constexpr int NCH = (1 << T) / EPC / NT;
+    constexpr int CCH = (1 << T) / 16 / NT;
+    constexpr uint32_t HC = (1u << (T - 1)) / 16;  // cost chunks per half
+    const uint32_t tid = threadIdx.x;
+    if (state) {
+        char *dst = reinterpret_cast<char *>(buf) + 16 * tid;
+        const V *reg = st + base + EPC * tid;
+        const V *mir = st + mbase + EPC * tid;
+#pragma unroll
+        for (int j = 0; j < NCH; ++j) {
+            const V *src = j < NCH / 2 ? reg + (size_t)EPC * NT * j : mir + (size_t)EPC * NT * (j - NCH / 2);
+            cp_async16(dst + (size_t)16 * NT * j, src);
+        }
+    }
+    if (cost) {
+#pragma unroll
+        for (int j = 0; j < CCH; ++j) {
+            const uint32_t q = tid + NT * j;
+            const uint8_t *src = q < HC ? cs + base + 16 * q : cs + mbase + 16 * (q - HC);
+            cp_async16(sc + 16 * q, src);
+        }
+    }
+}
+
+// Whether every slot of instance blockIdx.y is clear (all threads take part).
+__device__ __forceinline__ bool flip_symmetric(const int *slots, int nslots) {
+    int bad = 0;
+    for (int i = threadIdx.x; i < nslots; i += blockDim.x) bad |= slots[(size_t)blockIdx.y * nslots + i];
+    return !__syncthreads_or(bad);
+}
+
 // Pairwise sum of NR values fed in index order (NR a power of two; the index
 // must be a compile-time constant after unrolling, so the levels stay in
 // registers): element r joins the partial sums of the completed blocks below it,

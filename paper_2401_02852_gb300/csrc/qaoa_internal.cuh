@@ -65,6 +65,7 @@ enum KernelKind {
     K_SERVE_SMALL,
     K_SAMPLE,
     K_FLIP_CHECK,
+    K_MIRROR,
     K_NUM_KINDS
 };
 // Call before / after a launch on `stream`.  `after` checks the launch status.

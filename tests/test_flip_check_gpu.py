@@ -76,3 +76,30 @@ def test_single_and_without_results(arith, n):
         st2, _, _ = api.evolve(n, cost, inst.m, g, b, dtype, flags=flags, want=False, stream=s)
         s.synchronize()
         assert torch.equal(st, st2)
+
+
+# one and two high groups, full, partial and top-only masks of the backward plan
+@pytest.mark.parametrize("dtype,n,p", [("c64", 14, 2), ("c64", 15, 1), ("c64", 18, 2), ("c64", 20, 3), ("c64", 21, 2),
+                                       ("c128", 13, 2), ("c128", 14, 1), ("c128", 19, 2)])
+def test_gradients_of_symmetric_and_other_tables(dtype, n, p):
+    N = 1 << n
+    where = [None, 1, N - 2]
+    inst, tabs = _tables(n, 4 * n, where)
+    g, b = gen.linear_ramp(p)
+    g = g + 0.1
+    tdt = torch.complex64 if dtype == "c64" else torch.complex128
+    work = tuple(torch.full((len(where), N), 7.0, dtype=tdt, device="cuda") for _ in range(2))
+    ps, dg, db = api.grad_batch(n, torch.from_numpy(tabs).cuda(), inst.m, g, b, dtype, work=work)
+    tol = 1e-6 * (1 + n * p) if dtype == "c64" else 1e-8
+    for i, t in enumerate(tabs):
+        rps, rdg, rdb = oracle.grad(n, t, g, b)
+        scale = max(np.max(np.abs(rdg)), np.max(np.abs(rdb)))
+        assert abs(ps[i] - rps) <= (1e-4 if dtype == "c64" else 1e-10) * rps
+        assert np.max(np.abs(dg[i] - rdg)) <= tol * scale and np.max(np.abs(db[i] - rdb)) <= tol * scale
+        # the sweep ends on |+>^n, in both halves
+        psi = work[0][i].cpu().numpy()
+        amp = 2.0 ** (-n / 2)
+        assert np.max(np.abs(psi - amp)) <= (2e-6 if dtype == "c64" else 4e-15) * (1 + n * p) * amp
+    if dtype == "c64" or n < 19:
+        lam = work[1][0]
+        assert torch.equal(lam, lam.flip(0))
