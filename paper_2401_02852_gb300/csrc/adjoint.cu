@@ -322,95 +322,6 @@ __global__ void __launch_bounds__(PT) mirror_kernel(V *psi, V *lam, int n, const
     }
 }
 
-// ---------------------------------------------------------------------------
-// Small n: the whole forward and reverse sweep of one instance per CTA, both
-// states resident in shared memory.  tables: FP64 exp(-i gamma_l c) [p][m+1];
-// coefs: (c, S) per layer.  out: [batch][1 + p][2] = (p_succ, norm), then
-// (mixer sum, phase sum) per layer.
-template <typename R>
-__global__ void __launch_bounds__(PT) small_grad_kernel(const uint8_t *costs, int n, int m, int p, const double *tables,
-                                                        const double *coefs, double *out) {
-    using V = typename Cx<R>::V;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const uint32_t N = 1u << n;
-    V *sp = reinterpret_cast<V *>(smem_raw);
-    V *sl = sp + N;
-    uint8_t *sc = reinterpret_cast<uint8_t *>(sl + N);
-    const size_t inst = blockIdx.x;
-    const uint8_t *cost = costs + (inst << n);
-    double *o = out + inst * 2 * (1 + p);
-    for (uint32_t x = threadIdx.x; x < N; x += PT) sc[x] = cost[x];
-    const R amp = (R)(1.0 / sqrt((double)N));
-    for (uint32_t x = threadIdx.x; x < N; x += PT) sp[x] = V{amp, (R)0};
-    __syncthreads();
-    for (int l = 0; l < p; ++l) {
-        const double *tb = tables + 2 * (size_t)l * (m + 1);
-        for (uint32_t x = threadIdx.x; x < N; x += PT) {
-            const int cx = min((int)sc[x], m);
-            const V ph{(R)tb[2 * cx], (R)tb[2 * cx + 1]};
-            sp[x] = cmul(sp[x], ph);
-        }
-        const R c = (R)coefs[2 * l], S = (R)coefs[2 * l + 1];
-        for (int j = 0; j < n; ++j) {
-            __syncthreads();
-            for (uint32_t g = threadIdx.x; g < N / 2; g += PT) {
-                const uint32_t x0 = ((g >> j) << (j + 1)) | (g & ((1u << j) - 1u)), x1 = x0 | (1u << j);
-                const V a = sp[x0], b = sp[x1];
-                sp[x0] = V{fma(c, a.x, -S * b.y), fma(c, a.y, S * b.x)};
-                sp[x1] = V{fma(c, b.x, -S * a.y), fma(c, b.y, S * a.x)};
-            }
-        }
-        __syncthreads();
-    }
-    double acc[2] = {0.0, 0.0};
-    for (uint32_t x = threadIdx.x; x < N; x += PT) {
-        const V v = sp[x];
-        const double w = (double)v.x * v.x + (double)v.y * v.y;
-        acc[1] += w;
-        const bool sol = sc[x] == 0;
-        if (sol) acc[0] += w;
-        sl[x] = sol ? v : V{(R)0, (R)0};
-    }
-    block_sum<2>(acc);
-    if (threadIdx.x == 0) {
-        o[0] = acc[0];
-        o[1] = acc[1];
-    }
-    for (int l = p - 1; l >= 0; --l) {
-        const R c = (R)coefs[2 * l], S = (R)coefs[2 * l + 1];
-        R term = 0;
-        for (int j = 0; j < n; ++j) {
-            __syncthreads();
-            for (uint32_t g = threadIdx.x; g < N / 2; g += PT) {
-                const uint32_t x0 = ((g >> j) << (j + 1)) | (g & ((1u << j) - 1u)), x1 = x0 | (1u << j);
-                V a = sp[x0], b = sp[x1], la = sl[x0], lb = sl[x1];
-                inv_pair(a, b, la, lb, c, S, term);
-                sp[x0] = a;
-                sp[x1] = b;
-                sl[x0] = la;
-                sl[x1] = lb;
-            }
-        }
-        __syncthreads();
-        const double *tb = tables + 2 * (size_t)l * (m + 1);
-        R gterm = 0;
-        for (uint32_t x = threadIdx.x; x < N; x += PT) {
-            const int cst = min((int)sc[x], m);
-            const V vp = sp[x], vl = sl[x];
-            gterm += (R)cst * (vl.x * vp.y - vl.y * vp.x);
-            const V ph{(R)tb[2 * cst], (R)(-tb[2 * cst + 1])};
-            sp[x] = cmul(vp, ph);
-            sl[x] = cmul(vl, ph);
-        }
-        double g2[2] = {(double)term, (double)gterm};
-        block_sum<2>(g2);
-        if (threadIdx.x == 0) {
-            o[2 * (1 + l)] = g2[0];
-            o[2 * (1 + l) + 1] = g2[1];
-        }
-    }
-}
-
 // Dynamic shared memory of a backward pass: the two tile buffers, then (low
 // pass, m >= 0) two cost-byte buffers and the phase table.
 template <typename R>
@@ -469,9 +380,6 @@ static int adj_init(AdjKernels<R> **out) {
                     e = cudaFuncSetAttribute(ks.fused[w][f], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)adj_smem<R>(MAX_TABLE - 1));
             }
-        const int small = (int)(2 * sizeof(typename Cx<R>::V) * (size_t(1) << Cx<R>::T) + (size_t(1) << Cx<R>::T));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(small_grad_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, small);
         if (e != cudaSuccess) return cuda_error(e, "adjoint kernel attributes");
         state[dev] = 1;
     }
@@ -591,48 +499,6 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
     return QAOA_OK;
 }
 
-template <typename R>
-static int grad_small(int batch, int n, const uint8_t *cost, int m, int p, const double *gamma, const double *beta,
-                      int flags, double *d_scr, double *h_scr, cudaStream_t stream, double *p_succ, double *dgamma,
-                      double *dbeta) {
-    AdjKernels<R> *ks = nullptr;
-    int rc = adj_init<R>(&ks);
-    if (rc) return rc;
-    const int sign = (flags & QAOA_MIXER_RX2B) ? -1 : 1;
-    const size_t tab_n = (size_t)p * (m + 1);
-    double *h_tab = h_scr;
-    double *h_coef = h_tab + 2 * tab_n;
-    for (int l = 0; l < p; ++l) {
-        for (int k = 0; k <= m; ++k) {
-            h_tab[2 * ((size_t)l * (m + 1) + k)] = std::cos(gamma[l] * k);
-            h_tab[2 * ((size_t)l * (m + 1) + k) + 1] = -std::sin(gamma[l] * k);
-        }
-        h_coef[2 * l] = std::cos(beta[l]);
-        h_coef[2 * l + 1] = sign * std::sin(beta[l]);
-    }
-    const size_t in_bytes = (2 * tab_n + 2 * (size_t)p) * sizeof(double);
-    double *d_tab = d_scr, *d_coef = d_scr + 2 * tab_n;
-    double *d_out = d_scr + 2 * tab_n + 2 * p;
-    const size_t out_n = (size_t)batch * 2 * (1 + p);
-    QAOA_CUDA_TRY(cudaMemcpyAsync(d_scr, h_scr, in_bytes, cudaMemcpyHostToDevice, stream));
-    const size_t smem = 2 * sizeof(typename Cx<R>::V) * (size_t(1) << n) + (size_t(1) << n);
-    profile_before(K_SMALL_N, stream);
-    small_grad_kernel<R><<<batch, PT, smem, stream>>>(cost, n, m, p, d_tab, d_coef, d_out);
-    if ((rc = profile_after(K_SMALL_N, stream))) return rc;
-    double *h_out = h_scr + 2 * tab_n + 2 * p;
-    QAOA_CUDA_TRY(cudaMemcpyAsync(h_out, d_out, out_n * sizeof(double), cudaMemcpyDeviceToHost, stream));
-    QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
-    for (int b = 0; b < batch; ++b) {
-        const double *o = h_out + (size_t)b * 2 * (1 + p);
-        if (p_succ) p_succ[b] = o[0];
-        for (int l = 0; l < p; ++l) {
-            dbeta[(size_t)b * p + l] = -2.0 * sign * o[2 * (1 + l)];
-            dgamma[(size_t)b * p + l] = 2.0 * o[2 * (1 + l) + 1];
-        }
-    }
-    return QAOA_OK;
-}
-
 static int grad_common(int batch, int n, const uint8_t *cost, int m, int p, const double *gamma, const double *beta,
                        int dtype, int flags, void *state, void *adj, double *p_succ, double *dgamma, double *dbeta,
                        void *stream_) {
@@ -651,15 +517,8 @@ static int grad_common(int batch, int n, const uint8_t *cost, int m, int p, cons
     cudaStream_t stream = (cudaStream_t)stream_;
     Scratch *sc = nullptr;
     int rc;
-    if (n <= small_n_limit(dtype)) {
-        const size_t words = 2 * (size_t)p * (m + 1) + 2 * (size_t)p + (size_t)batch * 2 * (1 + p) + 16;
-        if ((rc = scratch_for(stream, words * sizeof(double), words * sizeof(double), &sc))) return rc;
-        if (dtype == QAOA_C64)
-            return grad_small<float>(batch, n, cost, m, p, gamma, beta, flags, (double *)sc->dev, (double *)sc->host,
-                                     stream, p_succ, dgamma, dbeta);
-        return grad_small<double>(batch, n, cost, m, p, gamma, beta, flags, (double *)sc->dev, (double *)sc->host,
-                                  stream, p_succ, dgamma, dbeta);
-    }
+    if (n <= small_n_limit(dtype))
+        return grad_small(batch, n, cost, m, p, gamma, beta, dtype, flags, stream, p_succ, dgamma, dbeta);
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
     const int gxf = pass_grid_x(dtype, n - 1, batch);

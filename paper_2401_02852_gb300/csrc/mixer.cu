@@ -1,4 +1,4 @@
-// K2/K3/K4/K6: the QAOA layers U_B(beta) U_C(gamma) on a state in HBM.
+// K2/K3/K4: the QAOA layers U_B(beta) U_C(gamma) on a state in HBM.
 //
 //  * U_C(gamma) = diag(exp(-i gamma C(x))) (Eq. for U_C; Appendix A.3's
 //    diagonalisation): C(x) takes at most m + 1 values, so the phase is a lookup
@@ -549,169 +549,6 @@ __global__ void __launch_bounds__(PT) psucc_kernel(const typename Cx<R>::V *st, 
 }
 
 // ---------------------------------------------------------------------------
-// K6: whole evolution of one small instance per CTA, state resident in shared
-// memory.  Tables are FP64 complex [p][m+1] and coefficients [p][4]
-// (A, B, unit_a, unused) in device memory.
-template <typename R>
-__device__ __forceinline__ void smem_butterfly_pass(typename Cx<R>::V *s, int n, int j, int two, R A, R B,
-                                                    bool ua) {
-    using V = typename Cx<R>::V;
-    const uint32_t groups = 1u << (n - 1 - two);
-    for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) {
-        if (two) {
-            const uint32_t x0 = ((g >> j) << (j + 2)) | (g & ((1u << j) - 1u));
-            const uint32_t h1 = 1u << j, h2 = 2u << j;
-            V a = s[x0], b = s[x0 | h1], c = s[x0 | h2], d = s[x0 | h1 | h2];
-            if (ua) {
-                bfly<true>(a, b, A, B);
-                bfly<true>(c, d, A, B);
-                bfly<true>(a, c, A, B);
-                bfly<true>(b, d, A, B);
-            } else {
-                bfly<false>(a, b, A, B);
-                bfly<false>(c, d, A, B);
-                bfly<false>(a, c, A, B);
-                bfly<false>(b, d, A, B);
-            }
-            s[x0] = a;
-            s[x0 | h1] = b;
-            s[x0 | h2] = c;
-            s[x0 | h1 | h2] = d;
-        } else {
-            const uint32_t x0 = ((g >> j) << (j + 1)) | (g & ((1u << j) - 1u));
-            V a = s[x0], b = s[x0 | (1u << j)];
-            if (ua)
-                bfly<true>(a, b, A, B);
-            else
-                bfly<false>(a, b, A, B);
-            s[x0] = a;
-            s[x0 | (1u << j)] = b;
-        }
-    }
-}
-
-// Device conversions of FP64 inputs to each arithmetic (double-float: the
-// nearest float, then the nearest float to the remainder).
-template <typename R>
-__device__ __forceinline__ R real_dev(double x) {
-    if constexpr (is_df<R>()) {
-        const float hi = __double2float_rn(x);
-        return dfloat{hi, __double2float_rn(x - (double)hi)};
-    } else {
-        return (R)x;
-    }
-}
-template <typename R>
-__device__ __forceinline__ typename Cx<R>::V amp_dev(double re, double im) {
-    if constexpr (is_df<R>()) {
-        const dfloat r = real_dev<dfloat>(re), i = real_dev<dfloat>(im);
-        return make_float4(r.hi, r.lo, i.hi, i.lo);
-    } else {
-        typename Cx<R>::V z;
-        z.x = (R)re;
-        z.y = (R)im;
-        return z;
-    }
-}
-
-// One CTA per job: the whole evolution in shared memory.  complex128 runs in
-// FP64, or with QAOA_DF64 in double-float arithmetic (R = dfloat: float4
-// amplitudes in shared memory, FP64 (re, im) written out).
-template <typename R>
-__global__ void __launch_bounds__(PT) small_kernel(const SmallJob *jobs, const double *tables, const double *coefs,
-                                                   int max_n) {
-    using V = typename Cx<R>::V;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const SmallJob jb = jobs[blockIdx.x];
-    const int n = jb.n;
-    const uint32_t N = 1u << n;
-    V *s = reinterpret_cast<V *>(smem_raw);
-    V *stab = s + (1u << max_n);
-    uint8_t *sc = reinterpret_cast<uint8_t *>(stab + MAX_TABLE);
-    for (uint32_t x = threadIdx.x; x < N; x += blockDim.x) sc[x] = jb.cost[x];
-    for (int l = 0; l < jb.p; ++l) {
-        const double *tb = tables + 2 * ((size_t)jb.table_off + (size_t)l * (jb.m + 1));
-        __syncthreads();
-        for (int c = threadIdx.x; c <= jb.m; c += blockDim.x) stab[c] = amp_dev<R>(tb[2 * c], tb[2 * c + 1]);
-        __syncthreads();
-        for (uint32_t x = threadIdx.x; x < N; x += blockDim.x) s[x] = l == 0 ? stab[sc[x]] : cmul(s[x], stab[sc[x]]);
-        const double *cf = coefs + 4 * ((size_t)jb.coef_off + l);
-        const R A = real_dev<R>(cf[0]), B = real_dev<R>(cf[1]);
-        const bool ua = cf[2] != 0.0;
-        for (int j = 0; j < n; j += 2) {
-            __syncthreads();
-            smem_butterfly_pass<R>(s, n, j, (j + 1 < n) ? 1 : 0, A, B, ua);
-        }
-    }
-    if (jb.p == 0) {  // |+>: the table of "layer 0" holds the amplitude
-        const double *tb = tables + 2 * (size_t)jb.table_off;
-        const V z = amp_dev<R>(tb[0], tb[1]);
-        for (uint32_t x = threadIdx.x; x < N; x += blockDim.x) s[x] = z;
-    }
-    __syncthreads();
-    double acc[2] = {0.0, 0.0};
-    for (uint32_t x = threadIdx.x; x < N; x += blockDim.x) {
-        const V v = s[x];
-        double w;
-        if constexpr (is_df<R>()) {
-            w = amp_prob(v);
-            if (jb.state)
-                reinterpret_cast<double2 *>(jb.state)[x] =
-                    make_double2((double)v.x + (double)v.y, (double)v.z + (double)v.w);
-        } else {
-            w = (double)v.x * (double)v.x + (double)v.y * (double)v.y;
-            if (jb.state) reinterpret_cast<V *>(jb.state)[x] = v;
-        }
-        acc[1] += w;
-        if (sc[x] == 0) acc[0] += w;
-    }
-    block_sum<2>(acc);
-    if (threadIdx.x == 0 && jb.result) {
-        jb.result[0] = acc[0];
-        jb.result[1] = acc[1];
-    }
-}
-
-int small_n_limit(int dtype) { return dtype == QAOA_C64 ? Cx<float>::T : Cx<double>::T; }
-int small_n_pack_limit(int dtype) { return dtype == QAOA_C64 ? 14 : 13; }
-
-static size_t small_smem(int dtype, int max_n) {
-    const size_t es = dtype == QAOA_C64 ? sizeof(float2) : sizeof(double2);
-    return es * ((size_t(1) << max_n) + MAX_TABLE) + (size_t(1) << max_n);
-}
-
-int launch_small_batch(int dtype, int n_jobs, const SmallJob *d_jobs, const double *d_tables, const double *d_coefs,
-                       int max_n, int flags, cudaStream_t stream) {
-    const size_t smem = small_smem(dtype, max_n);
-    {
-        static std::mutex mu;
-        static int state[MAX_DEVICES] = {};  // per device: 0 = not yet, 1 = ok
-        const int dev = current_device_slot();
-        if (dev < 0) return QAOA_ECUDA;
-        std::lock_guard<std::mutex> lk(mu);
-        if (!state[dev]) {
-            const int big = (int)small_smem(QAOA_C128, small_n_pack_limit(QAOA_C128));
-            cudaError_t e = cudaFuncSetAttribute(small_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)small_smem(QAOA_C64, small_n_pack_limit(QAOA_C64)));
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(small_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(small_kernel<dfloat>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-            if (e != cudaSuccess) return cuda_error(e, "small_kernel attributes");
-            state[dev] = 1;
-        }
-    }
-    profile_before(K_SMALL_N, stream);
-    if (dtype == QAOA_C64)
-        small_kernel<float><<<n_jobs, PT, smem, stream>>>(d_jobs, d_tables, d_coefs, max_n);
-    else if (flags & QAOA_DF64)
-        small_kernel<dfloat><<<n_jobs, PT, smem, stream>>>(d_jobs, d_tables, d_coefs, max_n);
-    else
-        small_kernel<double><<<n_jobs, PT, smem, stream>>>(d_jobs, d_tables, d_coefs, max_n);
-    return profile_after(K_SMALL_N, stream);
-}
-
-// ---------------------------------------------------------------------------
 // Host side of the multi-pass evolution.
 
 // Dynamic shared memory of a pass: the tile buffer, two cost-byte buffers and
@@ -903,7 +740,7 @@ template <typename R>
 static void fill_table(PhaseTab<R, MAX_TABLE> *tab, const EvolveReq &r, int l, int sign) {
     std::vector<double> re(r.m + 1), im(r.m + 1);
     const LayerCoef k = r.p > 0 ? layer_coef(r.beta[l], sign, arith_of(r.dtype, r.flags)) : LayerCoef{1.0, 1.0, 0.0, true};
-    double scale = std::pow(k.sigma, r.n);
+    double scale = layer_scale(k, r.n);
     if (l == 0) scale *= std::pow(2.0, -0.5 * r.n);
     phase_table(r.p > 0 ? r.gamma[l] : 0.0, scale, r.m, re.data(), im.data());
     for (int c = 0; c <= r.m; ++c) tab->t[c] = amp_from(&tab->t[c], re[c], im[c]);
@@ -1056,55 +893,6 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
     return rc;
 }
 
-// Small-n path of evolve_device: tables and coefficients through scratch.
-static int evolve_small(const EvolveReq &r, Scratch *sc, size_t off, cudaStream_t stream) {
-    const int sign = (r.flags & QAOA_MIXER_RX2B) ? -1 : 1;
-    const int pl = r.p > 0 ? r.p : 1;
-    const size_t tab_n = (size_t)pl * (r.m + 1);
-    char *hb = reinterpret_cast<char *>(sc->host) + off;
-    char *db = reinterpret_cast<char *>(sc->dev) + off;
-    double *h_tab = reinterpret_cast<double *>(hb);
-    double *h_coef = h_tab + 2 * tab_n;
-    SmallJob *h_jobs = reinterpret_cast<SmallJob *>(h_coef + 4 * pl);
-    std::vector<double> re(r.m + 1), im(r.m + 1);
-    for (int l = 0; l < pl; ++l) {
-        LayerCoef k = r.p > 0 ? layer_coef(r.beta[l], sign, arith_of(r.dtype, r.flags)) : LayerCoef{1.0, 1.0, 0.0, true};
-        double scale = std::pow(k.sigma, r.n);
-        if (l == 0) scale *= std::pow(2.0, -0.5 * r.n);
-        phase_table(r.p > 0 ? r.gamma[l] : 0.0, scale, r.m, re.data(), im.data());
-        for (int c = 0; c <= r.m; ++c) {
-            h_tab[2 * ((size_t)l * (r.m + 1) + c)] = re[c];
-            h_tab[2 * ((size_t)l * (r.m + 1) + c) + 1] = im[c];
-        }
-        h_coef[4 * l] = k.A;
-        h_coef[4 * l + 1] = k.B;
-        h_coef[4 * l + 2] = k.unit_a ? 1.0 : 0.0;
-        h_coef[4 * l + 3] = 0.0;
-    }
-    const size_t es = r.dtype == QAOA_C64 ? 8 : 16;
-    for (int b = 0; b < r.batch; ++b) {
-        SmallJob j;
-        j.cost = r.cost + ((size_t)b << r.n);
-        j.state = reinterpret_cast<char *>(r.state) + ((size_t)b << r.n) * es;
-        j.result = r.d_result ? r.d_result + 2 * b : nullptr;
-        j.n = r.n;
-        j.m = r.m;
-        j.p = r.p;
-        j.table_off = 0;
-        j.coef_off = 0;
-        h_jobs[b] = j;
-    }
-    const size_t bytes = (2 * tab_n + 4 * (size_t)pl) * sizeof(double) + (size_t)r.batch * sizeof(SmallJob);
-    QAOA_CUDA_TRY(cudaMemcpyAsync(db, hb, bytes, cudaMemcpyHostToDevice, stream));
-    int rc = launch_small_batch(r.dtype, r.batch, reinterpret_cast<SmallJob *>(db + (2 * tab_n + 4 * pl) * sizeof(double)),
-                                reinterpret_cast<double *>(db), reinterpret_cast<double *>(db) + 2 * tab_n, r.n, r.flags,
-                                stream);
-    if (rc) return rc;
-    // the pinned staging block is reused by the next call on this stream
-    QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
-    return QAOA_OK;
-}
-
 // Validates an evolution request (shared by the ABI entry points).
 static int validate_evolve(int batch, int n, const uint8_t *cost, int m, int p, const double *gamma,
                            const double *beta, int dtype, void *state) {
@@ -1156,18 +944,14 @@ static int evolve_common(int batch, int n, const uint8_t *d_cost, int m, int p, 
     EvolveReq r{batch, n, m, p, dtype, flags, d_cost, d_state, adj, gamma, beta, nullptr};
     Scratch *sc = nullptr;
     if (n <= small_n_limit(dtype) && !adj) {
-        const int pl = p > 0 ? p : 1;
-        const size_t stage = (2 * (size_t)pl * (m + 1) + 4 * (size_t)pl) * sizeof(double) +
-                             (size_t)batch * sizeof(SmallJob) + 256;
-        const size_t res = (size_t)batch * 2 * sizeof(double);
-        rc = scratch_for(stream, stage + res, stage + res, &sc);
+        const size_t stage = (small_stage_bytes(dtype, m, p) + 255) & ~(size_t)255, res = (size_t)batch * 2 * sizeof(double);
+        rc = scratch_for(stream, stage, stage + res, &sc);
         if (rc) return rc;
-        if (want) r.d_result = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->dev) + stage);
-        rc = evolve_small(r, sc, 0, stream);
-        if (rc || !want) return rc;
+        // the kernel writes its results into the pinned block itself
         double *h = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->host) + stage);
-        QAOA_CUDA_TRY(cudaMemcpyAsync(h, r.d_result, res, cudaMemcpyDeviceToHost, stream));
-        QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
+        if (want) r.d_result = h;
+        rc = evolve_small(r, sc->host, sc->dev, stream);
+        if (rc || !want) return rc;
         for (int b = 0; b < batch; ++b) {
             if (p_succ) p_succ[b] = h[2 * b];
             if (norm) norm[b] = h[2 * b + 1];

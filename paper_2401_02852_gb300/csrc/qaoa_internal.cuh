@@ -138,7 +138,12 @@ enum Arith { ARITH_F32 = 0, ARITH_F64 = 1, ARITH_DF = 2 };
 struct LayerCoef {
     double sigma, A, B;
     bool unit_a;  // true: A == 1, else B == 1
+    double s2 = 1.0, s2_lo = 0.0;  // 1 / sigma^2 = s2 + s2_lo (beyond FP64)
 };
+// sigma^n and sigma^2, each within an ulp or two: the n-th power of a rounded
+// sigma is off by n roundings, the same on every amplitude of a layer.
+double layer_scale(const LayerCoef &k, int n);
+double layer_sigma2(const LayerCoef &k);
 LayerCoef layer_coef(double beta, int sign, int arith);
 inline int arith_of(int dtype, int flags) {
     return dtype == QAOA_C64 ? ARITH_F32 : ((flags & QAOA_DF64) ? ARITH_DF : ARITH_F64);
@@ -218,8 +223,26 @@ struct SmallJob {
     int table_off;        // offset (in complex entries) of this job's tables
     int coef_off;         // offset (in layers) of this job's coefficients
 };
-int launch_small_batch(int dtype, int n_jobs, const SmallJob *d_jobs, const double *d_tables,
-                       const double *d_coefs, int max_n, int flags, cudaStream_t stream);
+// Tables and coefficients are in the kernel's own types (small_fill_layers:
+// small_entry_bytes per table entry, small_coef_bytes per layer, 16-byte aligned).
+// A job's arithmetic and sums depend on its own inputs only, whatever it is
+// packed with.
+size_t small_entry_bytes(int dtype);
+size_t small_coef_bytes(int dtype);
+void small_fill_layers(int dtype, int flags, int n, int m, int p, const double *gamma, const double *beta, void *tab,
+                       void *coef);
+int launch_small_batch(int dtype, int n_jobs, const SmallJob *d_jobs, const void *d_tables, const void *d_coefs,
+                       int max_n, int flags, cudaStream_t stream);
+// The evolutions of r (n at most small_n_limit) through the same kernel;
+// r.d_result may be pinned host memory.  Tables too long for kernel parameters
+// are staged: small_stage_bytes on the host (pinned) and the device.  Waits for
+// the stream when it staged them or r.d_result is set.
+size_t small_stage_bytes(int dtype, int m, int p);
+int evolve_small(const EvolveReq &r, void *h_stage, void *d_stage, cudaStream_t stream);
+// Gradients for n at most small_n_limit (through the stream's scratch).  Waits
+// for the stream.
+int grad_small(int batch, int n, const uint8_t *cost, int m, int p, const double *gamma, const double *beta, int dtype,
+               int flags, cudaStream_t stream, double *p_succ, double *dgamma, double *dbeta);
 // Largest n that the single-instance evolution runs in one CTA (the pass path
 // needs n > T), and the largest n the packed small-n kernel accepts.
 int small_n_limit(int dtype);

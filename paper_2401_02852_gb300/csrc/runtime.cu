@@ -289,6 +289,20 @@ static double coef_in_arith(double x, int arith) {
     return x;
 }
 
+// 1 + x^2, |x| <= 1, as s2 + s2_lo: Fast2Sum of 1 and the FMA form of Dekker's product.
+static void one_plus_square(double x, LayerCoef *k) {
+    const double q = x * x, e = std::fma(x, x, -q);
+    k->s2 = 1.0 + q;
+    k->s2_lo = (q - (k->s2 - 1.0)) + e;
+}
+
+double layer_scale(const LayerCoef &k, int n) {
+    const double s = std::pow(k.s2, -0.5 * n) * (1.0 - 0.5 * n * (k.s2_lo / k.s2));
+    return k.sigma < 0.0 && (n & 1) ? -s : s;
+}
+
+double layer_sigma2(const LayerCoef &k) { return (1.0 - k.s2_lo / k.s2) / k.s2; }
+
 LayerCoef layer_coef(double beta, int sign, int arith) {
     const double c = std::cos(beta), sn = std::sin(beta);
     const double S = sign * sn;  // butterfly: a' = c a + i S b, b' = i S a + c b
@@ -301,12 +315,14 @@ LayerCoef layer_coef(double beta, int sign, int arith) {
     if (std::fabs(c) >= std::fabs(S)) {
         k.A = 1.0;
         k.B = coef_in_arith(S / c, arith);
-        k.sigma = std::copysign(1.0 / std::sqrt(1.0 + k.B * k.B), c);
+        one_plus_square(k.B, &k);
+        k.sigma = std::copysign(1.0 / std::sqrt(k.s2), c);
         k.unit_a = true;
     } else {
         k.A = coef_in_arith(c / S, arith);
         k.B = 1.0;
-        k.sigma = std::copysign(1.0 / std::sqrt(1.0 + k.A * k.A), S);
+        one_plus_square(k.A, &k);
+        k.sigma = std::copysign(1.0 / std::sqrt(k.s2), S);
         k.unit_a = false;
     }
     return k;

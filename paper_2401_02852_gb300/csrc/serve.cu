@@ -263,8 +263,6 @@ static int launch_group(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<Re
 // Launch a packed batch of small requests on slot s.
 static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<Req>> &batch) {
     const int B = (int)batch.size();
-    const int sign = (sv->o.flags & QAOA_MIXER_RX2B) ? -1 : 1;
-    const int arith = arith_of(sv->o.dtype, sv->o.flags);
     int m_stride = 1, max_n = 1;
     size_t tab_n = 0, coef_n = 0, cost_bytes = 0;
     for (auto &q : batch) {
@@ -280,8 +278,9 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
     const size_t o_n = align(o_m + (size_t)B * sizeof(int));
     const size_t o_off = align(o_n + (size_t)B * sizeof(int));
     const size_t o_tab = align(o_off + (size_t)B * sizeof(uint64_t));
-    const size_t o_coef = align(o_tab + 2 * tab_n * sizeof(double));
-    const size_t o_jobs = align(o_coef + 4 * coef_n * sizeof(double));
+    const size_t eb = small_entry_bytes(sv->o.dtype), cb = small_coef_bytes(sv->o.dtype);
+    const size_t o_coef = align(o_tab + eb * tab_n);
+    const size_t o_jobs = align(o_coef + cb * coef_n);
     const size_t o_up = align(o_jobs + (size_t)B * sizeof(SmallJob));  // end of the uploaded part
     const size_t o_stats = o_up;
     const size_t o_res = align(o_stats + (size_t)B * 2 * sizeof(unsigned long long));
@@ -294,11 +293,8 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
     int *h_m = reinterpret_cast<int *>(h + o_m);
     int *h_n = reinterpret_cast<int *>(h + o_n);
     uint64_t *h_off = reinterpret_cast<uint64_t *>(h + o_off);
-    double *h_tab = reinterpret_cast<double *>(h + o_tab);
-    double *h_coef = reinterpret_cast<double *>(h + o_coef);
     SmallJob *h_jobs = reinterpret_cast<SmallJob *>(h + o_jobs);
     size_t toff = 0, coff = 0, boff = 0;
-    std::vector<double> re, im;
     for (int b = 0; b < B; ++b) {
         Req &q = *batch[b];
         naesat_instance inst{q.n, q.m, q.k, q.var.data(), q.neg.data()};
@@ -308,22 +304,8 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
         h_off[b] = boff;
         const int pl = std::max(q.p, 1);
         const int mt = table_top(q.m);
-        re.resize(mt + 1);
-        im.resize(mt + 1);
-        for (int l = 0; l < pl; ++l) {
-            LayerCoef k = q.p > 0 ? layer_coef(q.beta[l], sign, arith) : LayerCoef{1.0, 1.0, 0.0, true};
-            double scale = std::pow(k.sigma, q.n);
-            if (l == 0) scale *= std::pow(2.0, -0.5 * q.n);
-            phase_table(q.p > 0 ? q.gamma[l] : 0.0, scale, mt, re.data(), im.data());
-            for (int c = 0; c <= mt; ++c) {
-                h_tab[2 * (toff + (size_t)l * (mt + 1) + c)] = re[c];
-                h_tab[2 * (toff + (size_t)l * (mt + 1) + c) + 1] = im[c];
-            }
-            h_coef[4 * (coff + l)] = k.A;
-            h_coef[4 * (coff + l) + 1] = k.B;
-            h_coef[4 * (coff + l) + 2] = k.unit_a ? 1.0 : 0.0;
-            h_coef[4 * (coff + l) + 3] = 0.0;
-        }
+        small_fill_layers(sv->o.dtype, sv->o.flags, q.n, mt, q.p, q.gamma.data(), q.beta.data(), h + o_tab + eb * toff,
+                          h + o_coef + cb * coff);
         SmallJob j;
         j.cost = reinterpret_cast<const uint8_t *>(s.d_cost) + boff;
         j.state = nullptr;
@@ -346,7 +328,7 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
                                       s.stream, true)))
         return rc;
     if ((rc = launch_small_batch(sv->o.dtype, B, reinterpret_cast<SmallJob *>(d + o_jobs),
-                                 reinterpret_cast<double *>(d + o_tab), reinterpret_cast<double *>(d + o_coef), max_n,
+                                 d + o_tab, d + o_coef, max_n,
                                  sv->o.flags, s.stream)))
         return rc;
     QAOA_CUDA_TRY(cudaMemcpyAsync(h + o_stats, d + o_stats, total - o_stats, cudaMemcpyDeviceToHost, s.stream));
