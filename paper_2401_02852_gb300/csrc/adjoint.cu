@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
             stab[i] = i <= a.m ? tab.t[i] : z;
         }
     }
+    pdl_wait();
     const bool half = flip_symmetric(a.slots, a.nslots);
     if constexpr (!LOW)
         adj_tiles<R, LOW, MODE, HROW, FULL, false>(a, half, tp, scs, stab);
@@ -312,6 +313,7 @@ __global__ void __launch_bounds__(PT, sizeof(R) == 4 ? 2 : 1) adj_kernel(const _
 // backward sweep is done: element x goes to its complement N - 1 - x.
 template <typename V>
 __global__ void __launch_bounds__(PT) mirror_kernel(V *psi, V *lam, int n, const int *slots, int nslots) {
+    pdl_wait();
     if (!flip_symmetric(slots, nslots)) return;
     const size_t N = (size_t)1 << n, off = (size_t)blockIdx.y << n;
     psi += off;
@@ -456,9 +458,9 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
             if (L.mode == A_FUSED) return set_error(QAOA_ECUDA, "adjoint schedule: fused low pass");
             profile_before(K_ADJ_LOW, stream);
             if (L.mode == A_PHASE)
-                ks->low_phase<<<dim3(gxa, batch), PT, adj_smem<R>(m), stream>>>(a, *tab);
+                launch_pdl(ks->low_phase, dim3(gxa, batch), dim3(PT), adj_smem<R>(m), stream, a, *tab);
             else
-                ks->low<<<dim3(gxa, batch), PT, adj_smem<R>(-1), stream>>>(a, none);
+                launch_pdl(ks->low, dim3(gxa, batch), dim3(PT), adj_smem<R>(-1), stream, a, none);
             rc = profile_after(K_ADJ_LOW, stream);
         } else {
             a.row = ps.row;
@@ -472,16 +474,17 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
             const int full = ps.bits == pl.tile_bits - ps.row ? 1 : (ps.bits <= AGeo<R>::RB ? 2 : 0);
             profile_before(K_ADJ_HIGH, stream);
             if (L.mode == A_PLAIN)
-                ks->high[wide][full]<<<dim3(gxa, batch), PT, adj_smem<R>(-1), stream>>>(a, none);
+                launch_pdl(ks->high[wide][full], dim3(gxa, batch), dim3(PT), adj_smem<R>(-1), stream, a, none);
             else  // A_FUSED, or A_PHASE as the fused kernel with an identity second layer
-                ks->fused[wide][full]<<<dim3(gxa, batch), PT, adj_smem<R>(m), stream>>>(a, *tab);
+                launch_pdl(ks->fused[wide][full], dim3(gxa, batch), dim3(PT), adj_smem<R>(m), stream, a, *tab);
             rc = profile_after(K_ADJ_HIGH, stream);
         }
         if (rc) return rc;
     }
     profile_before(K_MIRROR, stream);
-    mirror_kernel<V><<<dim3((unsigned)std::min<uint64_t>(1ull << (n - 9), (uint64_t)di.sms * 8 / batch + 1), batch), PT, 0,
-                       stream>>>(reinterpret_cast<V *>(state), reinterpret_cast<V *>(adj), n, d_slots, nslots);
+    const unsigned gxm = (unsigned)std::min<uint64_t>(1ull << (n - 9), (uint64_t)di.sms * 8 / batch + 1);
+    launch_pdl(mirror_kernel<V>, dim3(gxm, batch), dim3(PT), 0, stream, reinterpret_cast<V *>(state),
+               reinterpret_cast<V *>(adj), n, d_slots, nslots);
     if ((rc = profile_after(K_MIRROR, stream))) return rc;
     if ((rc = launch_reduce(d_apart, batch * p, gxa, 2, d_ares, stream))) return rc;
     QAOA_CUDA_TRY(cudaMemcpyAsync(h_scr, d_fres, (size_t)batch * 2 * sizeof(double), cudaMemcpyDeviceToHost, stream));

@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_con
         srec[i] = make_uint4(r.hi_mask, r.hi_neg, r.all_true, r.all_false);
     }
     __syncthreads();
+    pdl_wait();
     cost_table_body<NPL_SMALL>(prm.n, prm.m, srec, alive, &acount, cost, stats, prm.mirror != 0);
 }
 
@@ -336,6 +337,7 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, con
     __shared__ uint4 srec[CT_CHUNK];
     __shared__ uint4 alive[CT_CHUNK];
     __shared__ int acount;
+    pdl_wait();
     const int inst = blockIdx.y;
     const int m = ms[inst];
     const ClauseRec *g = recs + (size_t)inst * m_stride;
@@ -416,11 +418,11 @@ int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d
     const int mi = mirror ? 1 : 0;
     profile_before(K_COST_TABLE, stream);
     if (m_stride <= CT_PARAM_M)
-        cost_table_batch_kernel<NPL_SMALL><<<dim3(gx, batch), CT_THREADS, 0, stream>>>(n, d_ns, d_offs, d_recs, d_m,
-                                                                                     m_stride, d_costs, d_stats, mi);
+        launch_pdl(cost_table_batch_kernel<NPL_SMALL>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
+                   m_stride, d_costs, d_stats, mi);
     else
-        cost_table_batch_kernel<NPL_LARGE><<<dim3(gx, batch), CT_THREADS, 0, stream>>>(n, d_ns, d_offs, d_recs, d_m,
-                                                                                     m_stride, d_costs, d_stats, mi);
+        launch_pdl(cost_table_batch_kernel<NPL_LARGE>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
+                   m_stride, d_costs, d_stats, mi);
     return profile_after(K_COST_TABLE, stream);
 }
 
@@ -451,7 +453,7 @@ int launch_cost_table_one(const naesat_instance *inst, uint8_t *d_cost, unsigned
     const int gx = grid_for(words, 1);
     if (gx < 0) return QAOA_ECUDA;
     profile_before(K_COST_TABLE, stream);
-    cost_table_kernel<<<gx, CT_THREADS, 0, stream>>>(*prm, d_cost, d_stats);
+    launch_pdl(cost_table_kernel, dim3(gx), dim3(CT_THREADS), 0, stream, *prm, d_cost, d_stats);
     return profile_after(K_COST_TABLE, stream);
 }
 

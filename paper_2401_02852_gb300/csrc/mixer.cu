@@ -67,6 +67,7 @@ enum SymMode {
 // amplitudes; at small n by its launch.
 constexpr int CHECK_PT = 512;
 __global__ void __launch_bounds__(CHECK_PT) flip_check_kernel(const uint8_t *cost, int n, int *slots) {
+    pdl_wait();
     const uint4 *c = reinterpret_cast<const uint4 *>(cost + ((size_t)blockIdx.y << n));
     const uint32_t W = 1u << (n - 4), H = W / 2, step = gridDim.x * CHECK_PT;
     uint32_t bad = 0;
@@ -485,6 +486,7 @@ __global__ void __launch_bounds__(Cx<R>::PT, NB == 3 ? 1 : 2) pass_kernel(const 
         for (int i = threadIdx.x; i < 256 || i <= a.m; i += Cx<R>::PT) stab[i] = i <= a.m ? tab.t[i] : zero_amp<V>();
         __syncthreads();
     }
+    pdl_wait();
     bool half = SYM == SYM_HALF;
     if constexpr (SYM == SYM_CHECK) {
         if (a.slots) half = flip_symmetric(a.slots, a.nslots);
@@ -499,6 +501,7 @@ __global__ void __launch_bounds__(Cx<R>::PT, NB == 3 ? 1 : 2) pass_kernel(const 
 
 // Fixed-order reduction of per-block partials: out[b][k] = sum_j part[b][j][k].
 __global__ void __launch_bounds__(PT) reduce_partials_kernel(const double *part, int nblk, int nv, double *out) {
+    pdl_wait();
     const size_t b = blockIdx.x;
     double x[4] = {0, 0, 0, 0};
     for (int j = threadIdx.x; j < nblk; j += PT)
@@ -510,7 +513,7 @@ __global__ void __launch_bounds__(PT) reduce_partials_kernel(const double *part,
 
 int launch_reduce(const double *part, int groups, int nblk, int nv, double *out, cudaStream_t stream) {
     profile_before(K_REDUCE, stream);
-    reduce_partials_kernel<<<groups, PT, 0, stream>>>(part, nblk, nv, out);
+    launch_pdl(reduce_partials_kernel, dim3(groups), dim3(PT), 0, stream, part, nblk, nv, out);
     return profile_after(K_REDUCE, stream);
 }
 
@@ -521,6 +524,7 @@ __global__ void __launch_bounds__(PT) psucc_kernel(const typename Cx<R>::V *st, 
     // elements per thread per chunk, summed pairwise in R (complex64: FP32,
     // relative error at most 7 u = 4.2e-7); chunks and threads in FP64
     constexpr int CH = 32;
+    pdl_wait();
     const uint64_t N = 1ull << n;
     const uint64_t chunk = (uint64_t)PT * CH;
     double acc[2] = {0.0, 0.0};
@@ -762,7 +766,7 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
     const bool check = SYM == SYM_CHECK && r.slots && r.p > 0;
     if (check) {
         profile_before(K_FLIP_CHECK, stream);
-        flip_check_kernel<<<dim3(r.nslots, r.batch), CHECK_PT, 0, stream>>>(r.cost, r.n, r.slots);
+        launch_pdl(flip_check_kernel, dim3(r.nslots, r.batch), dim3(CHECK_PT), 0, stream, r.cost, r.n, r.slots);
         rc = profile_after(K_FLIP_CHECK, stream);
         if (rc) return rc;
     }
@@ -839,12 +843,12 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
             auto launch_low = [&](const auto &ls, dim3 g, size_t sm_phase, size_t sm_plain) -> int {
                 if (L.mode == MODE_INIT) {
                     fill_table<R>(tab, r, 0, sign);
-                    (r.p == 0 ? ls.init0 : ls.init[u1])<<<g, block, sm_phase, stream>>>(a, *tab);
+                    launch_pdl(r.p == 0 ? ls.init0 : ls.init[u1], g, block, sm_phase, stream, a, *tab);
                 } else if (L.mode == MODE_PHASE) {
                     fill_table<R>(tab, r, L.la, sign);
-                    ls.phase[u1]<<<g, block, sm_phase, stream>>>(a, *tab);
+                    launch_pdl(ls.phase[u1], g, block, sm_phase, stream, a, *tab);
                 } else if (L.mode == MODE_PLAIN) {
-                    (a.reduce ? ls.plain_red[u1] : ls.plain[u1])<<<g, block, sm_plain, stream>>>(a, none);
+                    launch_pdl(a.reduce ? ls.plain_red[u1] : ls.plain[u1], g, block, sm_plain, stream, a, none);
                 } else {
                     return set_error(QAOA_ECUDA, "schedule: fused low pass");
                 }
@@ -869,19 +873,19 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
             if (L.mode == MODE_INIT) {
                 fill_table<R>(tab, r, 0, sign);
                 auto k = wide ? (full ? wn.init[u1] : wp.init[u1]) : (full ? hn.init[u1] : hp.init[u1]);
-                k<<<grid, block, smem_phase, stream>>>(a, *tab);
+                launch_pdl(k, grid, block, smem_phase, stream, a, *tab);
             } else if (L.mode == MODE_FUSED) {
                 fill_table<R>(tab, r, L.la + 1, sign);
                 auto k = wide ? (full ? wn.fused[u1][u2] : wp.fused[u1][u2])
                               : (full ? hn.fused[u1][u2] : hp.fused[u1][u2]);
                 const size_t smem_fused = pass_smem<R>(true, r.m, 1, early_landing<R, false, MODE_FUSED, 1>());
-                k<<<grid, block, smem_fused, stream>>>(a, *tab);
+                launch_pdl(k, grid, block, smem_fused, stream, a, *tab);
             } else if (L.mode == MODE_PLAIN) {
                 auto k = a.reduce ? (wide ? (full ? wn.plain_red[u1] : wp.plain_red[u1])
                                           : (full ? hn.plain_red[u1] : hp.plain_red[u1]))
                                   : (wide ? (full ? wn.plain[u1] : wp.plain[u1])
                                           : (full ? hn.plain[u1] : hp.plain[u1]));
-                k<<<grid, block, smem_plain, stream>>>(a, none);
+                launch_pdl(k, grid, block, smem_plain, stream, a, none);
             } else {
                 return set_error(QAOA_ECUDA, "schedule: phase-at-load on a strided pass");
             }
@@ -970,15 +974,14 @@ static int evolve_common(int batch, int n, const uint8_t *d_cost, int m, int p, 
         if ((rc = device_info(&di))) return rc;
         r.nslots = flip_slots(n, batch, di.sms);
     }
-    rc = scratch_for(stream, part + res + (size_t)batch * r.nslots * sizeof(int) + 256, res + 64, &sc);
+    rc = scratch_for(stream, part + (size_t)batch * r.nslots * sizeof(int) + 256, res + 64, &sc);
     if (rc) return rc;
     double *d_part = reinterpret_cast<double *>(sc->dev);
-    if (r.nslots) r.slots = reinterpret_cast<int *>(reinterpret_cast<char *>(sc->dev) + part + res);
-    if (want) r.d_result = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->dev) + part);
+    if (r.nslots) r.slots = reinterpret_cast<int *>(reinterpret_cast<char *>(sc->dev) + part);
+    double *h = reinterpret_cast<double *>(sc->host);
+    if (want) r.d_result = h;  // the reduction writes into the pinned block itself
     rc = evolve_device_impl(r, stream, d_part, gx);
     if (rc || !want) return rc;
-    double *h = reinterpret_cast<double *>(sc->host);
-    QAOA_CUDA_TRY(cudaMemcpyAsync(h, r.d_result, res, cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
     for (int b = 0; b < batch; ++b) {
         if (p_succ) p_succ[b] = scale * h[2 * b];
@@ -1027,13 +1030,13 @@ extern "C" int qaoa_success_prob(int n, const uint8_t *d_cost, const void *d_sta
     double *d_res = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->dev) + part);
     profile_before(K_PSUCC, stream);
     if (dtype == QAOA_C64)
-        psucc_kernel<float><<<grid, PT, 0, stream>>>(reinterpret_cast<const float2 *>(d_state), d_cost, n, d_part);
+        launch_pdl(psucc_kernel<float>, dim3(grid), dim3(PT), 0, stream, reinterpret_cast<const float2 *>(d_state), d_cost, n, d_part);
     else
-        psucc_kernel<double><<<grid, PT, 0, stream>>>(reinterpret_cast<const double2 *>(d_state), d_cost, n, d_part);
+        launch_pdl(psucc_kernel<double>, dim3(grid), dim3(PT), 0, stream, reinterpret_cast<const double2 *>(d_state), d_cost, n, d_part);
     rc = profile_after(K_PSUCC, stream);
     if (rc) return rc;
     profile_before(K_REDUCE, stream);
-    reduce_partials_kernel<<<1, PT, 0, stream>>>(d_part, grid, 2, d_res);
+    launch_pdl(reduce_partials_kernel, dim3(1), dim3(PT), 0, stream, d_part, grid, 2, d_res);
     rc = profile_after(K_REDUCE, stream);
     if (rc) return rc;
     double *h = reinterpret_cast<double *>(sc->host);
@@ -1099,13 +1102,13 @@ extern "C" int qaoa_success_prob_noalloc(int n, const uint8_t *d_cost, const voi
     double *d_res = scr + 2 * NOALLOC_MAX_BLOCKS;     // [2]
     profile_before(K_PSUCC, stream);
     if (dtype == QAOA_C64)
-        psucc_kernel<float><<<grid, PT, 0, stream>>>(reinterpret_cast<const float2 *>(d_state), d_cost, n, d_part);
+        launch_pdl(psucc_kernel<float>, dim3(grid), dim3(PT), 0, stream, reinterpret_cast<const float2 *>(d_state), d_cost, n, d_part);
     else
-        psucc_kernel<double><<<grid, PT, 0, stream>>>(reinterpret_cast<const double2 *>(d_state), d_cost, n, d_part);
+        launch_pdl(psucc_kernel<double>, dim3(grid), dim3(PT), 0, stream, reinterpret_cast<const double2 *>(d_state), d_cost, n, d_part);
     rc = profile_after(K_PSUCC, stream);  // counts the launch, checks its status
     if (rc) return rc;
     profile_before(K_REDUCE, stream);
-    reduce_partials_kernel<<<1, PT, 0, stream>>>(d_part, grid, 2, d_res);
+    launch_pdl(reduce_partials_kernel, dim3(1), dim3(PT), 0, stream, d_part, grid, 2, d_res);
     rc = profile_after(K_REDUCE, stream);
     if (rc) return rc;
     double h[2];  // pageable host copy: the runtime stages it, nothing is allocated here

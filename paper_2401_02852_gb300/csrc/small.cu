@@ -391,6 +391,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 2 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_bad;
     __shared__ double s_sum[2];
+    pdl_wait();
     SmallJob jb = all;
     if (jobs) {
         jb = jobs[blockIdx.x >> CB];
@@ -524,6 +525,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_bad;
     __shared__ double2 s_red[CB == 0 ? SMALL_PT : SMALL_PT_CL];
+    pdl_wait();
     const uint8_t *cost = costs + ((size_t)(blockIdx.x >> CB) << n);
     V *s = reinterpret_cast<V *>(smem_raw);
     V *sl = s + ((1u << n) >> CB);
@@ -699,12 +701,14 @@ static int launch_clusters(const void *kernel, int n_clusters, int cb, int threa
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1u << cb;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = 1u << cb;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = cb > 0 ? 1 : 0;
+    cfg.numAttrs = cb > 0 ? 2 : 1;
     QAOA_CUDA_TRY(cudaLaunchKernelExC(&cfg, kernel, args));
     return QAOA_OK;
 }
