@@ -45,15 +45,50 @@ def _np_ptr(a: np.ndarray) -> ctypes.c_void_p:
     return ctypes.c_void_p(a.ctypes.data) if a.size else ctypes.c_void_p(0)
 
 
+_I32, _U8 = np.dtype(np.int32), np.dtype(np.uint8)
+
+
+def _addr(a: np.ndarray) -> int:
+    """Address of a C-contiguous array's data, 0 when it is empty.  (Through the
+    buffer protocol, a third of the time of ndarray.ctypes; a read-only array
+    does not export a writable buffer.)"""
+    if not a.size:
+        return 0
+    try:
+        return ctypes.addressof(ctypes.c_char.from_buffer(a))
+    except TypeError:
+        return a.ctypes.data
+
+
+def _contiguous(a, dtype: np.dtype) -> np.ndarray:
+    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+        return a
+    return np.ascontiguousarray(a, dtype=dtype)
+
+
 class _Inst:
     """Keeps the numpy arrays alive while the C struct points at them."""
 
     def __init__(self, inst):
-        self.var = np.ascontiguousarray(inst.var, dtype=np.int32)
-        self.neg = np.ascontiguousarray(inst.neg, dtype=np.uint8)
+        self.var = _contiguous(inst.var, _I32)
+        self.neg = _contiguous(inst.neg, _U8)
         m = int(self.var.shape[0])
         k = int(self.var.shape[1]) if self.var.ndim == 2 else int(inst.k)
-        self.s = NaesatInstance(int(inst.n), m, k, _np_ptr(self.var).value or 0, _np_ptr(self.neg).value or 0)
+        self.s = NaesatInstance(int(inst.n), m, k, _addr(self.var), _addr(self.neg))
+
+
+_INSTANCE = np.dtype([("n", "i4"), ("m", "i4"), ("k", "i4"), ("var", "u8"), ("neg", "u8")], align=True)
+assert _INSTANCE.itemsize == ctypes.sizeof(NaesatInstance)
+
+
+def _instance_array(insts: Sequence):
+    """The C instances of a batch as one array, and the arrays it points to."""
+    keep, rows = [], []
+    for i in insts:
+        var, neg = _contiguous(i.var, _I32), _contiguous(i.neg, _U8)
+        keep.append((var, neg))
+        rows.append((i.n, len(var), var.shape[1] if var.ndim == 2 else i.k, _addr(var), _addr(neg)))
+    return np.array(rows, dtype=_INSTANCE), keep
 
 
 def cost_table(inst, out: Optional[torch.Tensor] = None, stream=None, stats: bool = True):
@@ -92,11 +127,11 @@ def cost_table_batch(insts: Sequence, out: Optional[torch.Tensor] = None, stream
     n = int(insts[0].n)
     if out is None:
         out = torch.empty((B, 1 << n), dtype=torch.uint8, device="cuda")
-    cis = [_Inst(i) for i in insts]
-    arr = (NaesatInstance * B)(*[c.s for c in cis])
+    arr, keep = _instance_array(insts)
     ns = np.zeros(B, dtype=np.uint64)
     mx = np.zeros(B, dtype=np.uint32)
-    check(load().naesat_cost_table_batch(B, ctypes.byref(arr), _ptr(out), _np_ptr(ns), _np_ptr(mx), _stream(stream)))
+    check(load().naesat_cost_table_batch(B, _np_ptr(arr), _ptr(out), _np_ptr(ns), _np_ptr(mx), _stream(stream)))
+    del keep
     return out, ns, mx
 
 

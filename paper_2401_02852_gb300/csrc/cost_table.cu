@@ -49,6 +49,7 @@ namespace qaoa {
 constexpr int CT_THREADS = 256;
 constexpr int CT_CHUNK = 1024;     // clause records staged in shared memory at a time
 constexpr int CT_PARAM_M = 1023;   // largest m passed as kernel parameters
+constexpr size_t ENCODE_MIN_LITS = 1 << 15;  // batches encoded on the device
 constexpr int NPL_SMALL = 10;      // bit planes for m <= 1023
 constexpr int NPL_LARGE = 13;      // bit planes for m <= 8191
 static_assert(QAOA_MAX_M < (1 << NPL_LARGE), "counts must fit the planes");
@@ -328,16 +329,20 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_con
 // at costs + inst 2^n; otherwise instance inst has ns[inst] qubits and its table
 // at costs + offs[inst].  Records of up to CT_CHUNK clauses are copied to
 // shared memory once; longer lists are read from global memory chunk by chunk.
+// `bad` (nullable): set when the encoder found an invalid literal; nothing is
+// written then.
 template <int NPL>
 __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, const int *ns, const uint64_t *offs,
                                                                       const ClauseRec *recs, const int *ms,
                                                                       int m_stride, uint8_t *costs,
-                                                                      unsigned long long *stats, int mirror) {
+                                                                      unsigned long long *stats, int mirror,
+                                                                      const unsigned long long *bad) {
     static_assert(sizeof(ClauseRec) == sizeof(uint4), "a clause record is one 16-byte load");
     __shared__ uint4 srec[CT_CHUNK];
     __shared__ uint4 alive[CT_CHUNK];
     __shared__ int acount;
     pdl_wait();
+    if (bad && *bad) return;
     const int inst = blockIdx.y;
     const int m = ms[inst];
     const ClauseRec *g = recs + (size_t)inst * m_stride;
@@ -355,8 +360,54 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, con
     cost_table_body<NPL>(ni, m, src, alive, &acount, dst, stats + 2 * inst, mirror != 0);
 }
 
+// Clause records of a batch, one clause per thread, from the literals in host
+// memory (HostLits: the caller's own arrays where the device can read pageable
+// memory through the host's page tables, a pinned copy elsewhere), with the
+// checks of validate_instance: *bad is set when a variable is outside [0, n), a
+// negation flag is not 0 or 1, or a variable is repeated.
+//
+// Bound by the reads over the chip-to-chip link.  The host's own loop over the
+// literals took 21 ms for 256 instances of about 3000 9-literal clauses (35 MB).
+struct HostLits {
+    const int32_t *var;
+    const uint8_t *neg;
+    int32_t m, k;
+};
+__global__ void __launch_bounds__(CT_THREADS) encode_kernel(int n, const HostLits *lits, int m_stride, ClauseRec *recs,
+                                                            unsigned long long *bad) {
+    pdl_wait();
+    const HostLits h = lits[blockIdx.y];
+    const int i = blockIdx.x * CT_THREADS + threadIdx.x;
+    bool wrong = false;
+    if (i < h.m) {
+        const int32_t *var = h.var + (size_t)i * h.k;
+        const uint8_t *neg = h.neg + (size_t)i * h.k;
+        uint32_t mask = 0, negp = 0, at = 0xFFFFFFFFu, af = 0xFFFFFFFFu;
+        for (int j = 0; j < h.k; ++j) {
+            const uint32_t v = (uint32_t)var[j], s = neg[j];
+            wrong |= v >= (uint32_t)n || s > 1u || ((mask >> (v & 31u)) & 1u);
+            mask |= 1u << (v & 31u);
+            negp |= (s & 1u) << (v & 31u);
+            if (v < 5) {  // bit b of the column: the literal is true at b
+                const uint32_t col = v == 0   ? 0xAAAAAAAAu
+                                     : v == 1 ? 0xCCCCCCCCu
+                                     : v == 2 ? 0xF0F0F0F0u
+                                     : v == 3 ? 0xFF00FF00u
+                                              : 0xFFFF0000u;
+                const uint32_t lit = s ? ~col : col;
+                at &= lit;
+                af &= ~lit;
+            }
+        }
+        *reinterpret_cast<uint4 *>(recs + (size_t)blockIdx.y * m_stride + i) =
+            make_uint4(mask & ~31u, negp & ~31u, at, af);
+    }
+    if (__syncthreads_or(wrong) && threadIdx.x == 0) *bad = 1;
+}
+
 // ---------------------------------------------------------------------------
-int validate_instance(const naesat_instance *inst) {
+// The sizes and pointers of an instance; its literals are checked apart.
+static int valid_sizes(const naesat_instance *inst) {
     if (!inst) return set_error(QAOA_EINVAL, "instance is NULL");
     const int n = inst->n, m = inst->m, k = inst->k;
     if (n < 1 || n > QAOA_MAX_N) return set_error(QAOA_ERANGE, "n=%d outside [1, %d]", n, QAOA_MAX_N);
@@ -364,6 +415,13 @@ int validate_instance(const naesat_instance *inst) {
     if (m == 0) return QAOA_OK;
     if (k < 1 || k > n) return set_error(QAOA_ERANGE, "k=%d outside [1, n=%d]", k, n);
     if (!inst->var || !inst->neg) return set_error(QAOA_EINVAL, "var/neg is NULL");
+    return QAOA_OK;
+}
+
+int validate_instance(const naesat_instance *inst) {
+    const int rc = valid_sizes(inst);
+    if (rc) return rc;
+    const int n = inst->n, m = inst->m, k = inst->k;
     for (int i = 0; i < m; ++i) {
         uint64_t seen = 0;
         for (int j = 0; j < k; ++j) {
@@ -411,7 +469,7 @@ static int grid_for(uint64_t words, int batch) {
 
 int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d_offs, const ClauseRec *d_recs,
                             const int *d_m, int m_stride, uint8_t *d_costs, unsigned long long *d_stats,
-                            cudaStream_t stream, bool mirror) {
+                            cudaStream_t stream, bool mirror, const unsigned long long *d_bad) {
     const uint64_t words = n >= 5 ? (1ull << (n - 5)) >> (mirror && n >= 6 ? 1 : 0) : 1ull;
     const int gx = grid_for(words, batch);
     if (gx < 0) return QAOA_ECUDA;
@@ -419,10 +477,10 @@ int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d
     profile_before(K_COST_TABLE, stream);
     if (m_stride <= CT_PARAM_M)
         launch_pdl(cost_table_batch_kernel<NPL_SMALL>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
-                   m_stride, d_costs, d_stats, mi);
+                   m_stride, d_costs, d_stats, mi, d_bad);
     else
         launch_pdl(cost_table_batch_kernel<NPL_LARGE>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
-                   m_stride, d_costs, d_stats, mi);
+                   m_stride, d_costs, d_stats, mi, d_bad);
     return profile_after(K_COST_TABLE, stream);
 }
 
@@ -502,37 +560,94 @@ extern "C" int naesat_cost_table_batch(int batch, const naesat_instance *insts, 
     if (batch < 1 || !insts || !d_costs) return set_error(QAOA_EINVAL, "batch/insts/d_costs");
     const int n = insts[0].n;
     int m_stride = 1;
+    size_t lits = 0;  // literals of the batch
     for (int b = 0; b < batch; ++b) {
-        int rc = validate_instance(&insts[b]);
+        int rc = valid_sizes(&insts[b]);
         if (rc) return rc;
         if (insts[b].n != n) return set_error(QAOA_EINVAL, "batch instances differ in n");
         m_stride = insts[b].m > m_stride ? insts[b].m : m_stride;
+        lits += insts[b].m > 0 ? (size_t)insts[b].m * insts[b].k : 0;
     }
+    // Short batches are checked and encoded here (about 3 ns a literal), without
+    // the encoder's launch and its first touch of the caller's memory.
+    const bool on_device = lits >= ENCODE_MIN_LITS && batch <= 65535;
+    if (!on_device)
+        for (int b = 0; b < batch; ++b) {
+            int rc = validate_instance(&insts[b]);
+            if (rc) return rc;
+        }
     cudaStream_t stream = (cudaStream_t)stream_;
-    const size_t rec_bytes = (size_t)batch * m_stride * sizeof(ClauseRec);
-    const size_t m_bytes = ((size_t)batch * sizeof(int) + 255) & ~(size_t)255;
-    const size_t stat_bytes = (size_t)batch * 2 * sizeof(unsigned long long);
+    DeviceInfo di;
+    int rc = device_info(&di);
+    if (rc) return rc;
+    auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    // device: records, clause counts, stats [batch][2] and the encoder's verdict,
+    // then its descriptors; host: the same, and a copy of the literals where the
+    // device cannot read them in place
+    const size_t rec_bytes = al((size_t)batch * m_stride * sizeof(ClauseRec));
+    const size_t m_bytes = al((size_t)batch * sizeof(int));
+    const size_t desc_bytes = on_device ? al((size_t)batch * sizeof(HostLits)) : 0;
+    const size_t stat_bytes = ((size_t)batch * 2 + 1) * sizeof(unsigned long long);
+    const bool copy = on_device && !di.pageable;
+    const size_t host_recs = on_device ? 0 : rec_bytes, copy_bytes = copy ? al(lits * 4) + lits : 0;
     Scratch *sc = nullptr;
-    int rc = scratch_for(stream, rec_bytes + m_bytes + stat_bytes + 512, rec_bytes + m_bytes + stat_bytes + 512, &sc);
+    rc = scratch_for(stream, rec_bytes + m_bytes + desc_bytes + stat_bytes,
+                     host_recs + m_bytes + desc_bytes + al(stat_bytes) + copy_bytes, &sc);
     if (rc) return rc;
     char *hbase = reinterpret_cast<char *>(sc->host);
     char *dbase = reinterpret_cast<char *>(sc->dev);
-    ClauseRec *h_recs = reinterpret_cast<ClauseRec *>(hbase);
-    int *h_m = reinterpret_cast<int *>(hbase + rec_bytes);
+    ClauseRec *d_recs = reinterpret_cast<ClauseRec *>(dbase);
+    int *d_m = reinterpret_cast<int *>(dbase + rec_bytes);
+    HostLits *d_lits = reinterpret_cast<HostLits *>(dbase + rec_bytes + m_bytes);
+    unsigned long long *d_stats = reinterpret_cast<unsigned long long *>(dbase + rec_bytes + m_bytes + desc_bytes);
+    unsigned long long *d_bad = on_device ? d_stats + 2 * (size_t)batch : nullptr;
+    char *h_up = hbase + host_recs;  // clause counts and descriptors, uploaded together
+    int *h_m = reinterpret_cast<int *>(h_up);
+    HostLits *h_lits = reinterpret_cast<HostLits *>(h_up + m_bytes);
+    unsigned long long *h_stats = reinterpret_cast<unsigned long long *>(h_up + m_bytes + desc_bytes);
+    char *h_copy = h_up + m_bytes + desc_bytes + al(stat_bytes);
+    size_t off = 0;
     for (int b = 0; b < batch; ++b) {
-        encode_instance(&insts[b], h_recs + (size_t)b * m_stride);
-        h_m[b] = insts[b].m;
+        const naesat_instance &q = insts[b];
+        h_m[b] = q.m;
+        if (!on_device) {
+            encode_instance(&q, reinterpret_cast<ClauseRec *>(hbase) + (size_t)b * m_stride);
+            continue;
+        }
+        HostLits &l = h_lits[b];
+        l = HostLits{q.var, q.neg, q.m, q.k};
+        if (copy && q.m > 0) {
+            const size_t c = (size_t)q.m * q.k;
+            int32_t *v = reinterpret_cast<int32_t *>(h_copy) + off;
+            uint8_t *g = reinterpret_cast<uint8_t *>(h_copy + al(lits * 4)) + off;
+            std::memcpy(v, q.var, c * sizeof(int32_t));
+            std::memcpy(g, q.neg, c);
+            l.var = v;
+            l.neg = g;
+            off += c;
+        }
     }
-    QAOA_CUDA_TRY(cudaMemcpyAsync(dbase, hbase, rec_bytes + m_bytes, cudaMemcpyHostToDevice, stream));
-    unsigned long long *d_stats = reinterpret_cast<unsigned long long *>(dbase + rec_bytes + m_bytes);
     QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, stat_bytes, stream));
-    rc = launch_cost_table_batch(batch, n, nullptr, nullptr, reinterpret_cast<const ClauseRec *>(dbase),
-                                 reinterpret_cast<const int *>(dbase + rec_bytes), m_stride, d_costs, d_stats, stream,
-                                 true);
+    if (on_device) {
+        QAOA_CUDA_TRY(cudaMemcpyAsync(d_m, h_up, m_bytes + desc_bytes, cudaMemcpyHostToDevice, stream));
+        profile_before(K_ENCODE, stream);
+        launch_pdl(encode_kernel, dim3((m_stride + CT_THREADS - 1) / CT_THREADS, batch), dim3(CT_THREADS), 0, stream, n,
+                   (const HostLits *)d_lits, m_stride, d_recs, d_bad);
+        if ((rc = profile_after(K_ENCODE, stream))) return rc;
+    } else {
+        QAOA_CUDA_TRY(cudaMemcpyAsync(dbase, hbase, rec_bytes + m_bytes, cudaMemcpyHostToDevice, stream));
+    }
+    rc = launch_cost_table_batch(batch, n, nullptr, nullptr, d_recs, d_m, m_stride, d_costs, d_stats, stream, true, d_bad);
     if (rc) return rc;
-    unsigned long long *h_stats = reinterpret_cast<unsigned long long *>(hbase + rec_bytes + m_bytes);
     QAOA_CUDA_TRY(cudaMemcpyAsync(h_stats, d_stats, stat_bytes, cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));  // the pinned staging block is reused by the next call
+    if (on_device && h_stats[2 * (size_t)batch]) {  // name the first invalid literal
+        for (int b = 0; b < batch; ++b) {
+            rc = validate_instance(&insts[b]);
+            if (rc) return rc;
+        }
+        return set_error(QAOA_EINVAL, "a literal changed during the call");
+    }
     int status = QAOA_OK;
     for (int b = 0; b < batch; ++b) {
         if (n_sol) n_sol[b] = h_stats[2 * b];

@@ -28,6 +28,7 @@ struct DeviceInfo {
     int device = -1;
     int sms = 0;
     size_t smem_optin = 0;
+    bool pageable = false;  // reads the host's pageable memory through its page tables
 };
 int device_info(DeviceInfo *out);
 
@@ -66,6 +67,7 @@ enum KernelKind {
     K_SAMPLE,
     K_FLIP_CHECK,
     K_MIRROR,
+    K_ENCODE,
     K_NUM_KINDS
 };
 // Call before / after a launch on `stream`.  `after` checks the launch status.
@@ -197,7 +199,7 @@ int encode_instance(const naesat_instance *inst, ClauseRec *out);
 int validate_instance(const naesat_instance *inst);
 // Launches the batched cost-table kernel: recs [batch][m_stride] on the device,
 // m per instance on the device, results into d_stats [batch][2] (uint64 n_sol,
-// uint64 max C) which must be zeroed first.  With d_ns == nullptr all
+// uint64 max C) which must be zeroed first; nothing is written when *d_bad is set.  With d_ns == nullptr all
 // instances have n qubits and consecutive tables; otherwise instance b has
 // d_ns[b] <= n qubits and its table at d_costs + d_offs[b].  `mirror`: the
 // tables are full ones (2^n entries), counted on their lower half and
@@ -205,7 +207,7 @@ int validate_instance(const naesat_instance *inst);
 // the halved state (n then counts their index bits).
 int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d_offs, const ClauseRec *d_recs,
                             const int *d_m, int m_stride, uint8_t *d_costs, unsigned long long *d_stats,
-                            cudaStream_t stream, bool mirror);
+                            cudaStream_t stream, bool mirror, const unsigned long long *d_bad = nullptr);
 // One table.  Up to 1023 clauses the records go as kernel parameters (no
 // staging); a longer list is copied to d_big (device, cost_table_big_bytes(m)
 // bytes, 16-byte aligned) and counted chunk by chunk.

@@ -46,6 +46,10 @@ int device_info(DeviceInfo *out) {
         int optin = 0;
         QAOA_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         d.smem_optin = (size_t)optin;
+        int pageable = 0, tables = 0;
+        QAOA_CUDA_TRY(cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev));
+        QAOA_CUDA_TRY(cudaDeviceGetAttribute(&tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev));
+        d.pageable = pageable && tables;
         it = g_devs.emplace(dev, d).first;
     }
     *out = it->second;
@@ -133,7 +137,7 @@ static thread_local cudaEvent_t t_pending = nullptr;
 
 static const char *k_names[K_NUM_KINDS] = {
     "cost_table", "pass_low", "pass_high", "small_n", "reduce",
-    "success_prob", "adjoint_low", "adjoint_high", "adjoint_seed", "serve_small", "sample", "flip_check", "mirror"};
+    "success_prob", "adjoint_low", "adjoint_high", "adjoint_seed", "serve_small", "sample", "flip_check", "mirror", "encode"};
 
 static cudaEvent_t take_event() {
     std::lock_guard<std::mutex> lk(g_prof_mu);
