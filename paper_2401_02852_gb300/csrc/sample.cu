@@ -16,9 +16,9 @@
 //      sets its scale E_g; each thread sums its entry's weights; an exact
 //      warp/block scan gives Q; the group total goes to FP64;
 //   2. block_prefix_kernel: inclusive prefix P of the group totals;
-//   3. draw_kernel: one warp per draw: a 32-way search over P (doubles >= +0
-//      compared as integers), the remainder in the group's units, a 32-way
-//      search over Q, then an integer warp scan over the entry's 32 weights.
+//   3. draw_kernel: four lanes per draw: a 4-way search over P (doubles >= +0
+//      compared as integers), the remainder in the group's units, a 4-way
+//      search over Q, then an integer scan over the entry's 32 weights.
 // The draws differ from a sequential FP64 scan of the probabilities only for
 // a u_j within about 2^-40 of a step of F (the weights' quantisation).
 // GB300's FP64 pipe is narrow: apart from a few operations per draw and per
@@ -39,7 +39,7 @@ constexpr int ENTRY_BITS = 5;    // log2 amplitudes per entry
 constexpr int GROUP_BITS = 8;    // log2 entries per group
 constexpr int GROUP = 1 << GROUP_BITS;
 constexpr int PREFIX_PT = 1024;  // threads of the group-prefix kernel
-constexpr int DRAW_WARPS = 8;    // draws per CTA of the draw kernel
+constexpr int DRAW_PT = 256;     // threads of the draw kernel, four per draw
 constexpr int W_TOP = 44;        // a group's largest probability scales into [2^44, 2^46)
 
 // Entry and group counts of a stored state of 2^ns amplitudes.
@@ -66,17 +66,6 @@ __host__ __device__ __forceinline__ uint64_t group_count(int ns) {
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }       // e in [-126, 127]
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// trunc(f) for |f| < 2^63 from the float's bits with integer operations (the
-// float-to-int64 conversion instruction runs on the FP64 pipe).
-__device__ __forceinline__ long long trunc_ll(float f) {
-    const uint32_t b = __float_as_uint(f);
-    const int ex = (int)((b >> 23) & 0xFFu);
-    const uint32_t mant = (b & 0x7FFFFFu) | (ex ? 0x800000u : 0u);
-    const int sh = (ex ? ex : 1) - 150;  // |f| = mant 2^sh
-    const long long v = sh >= 0 ? (long long)((unsigned long long)mant << sh) : (sh > -24 ? (long long)(mant >> -sh) : 0);
-    return (b >> 31) ? -v : v;
-}
-
 // trunc(v 2^E) for a double v from its bits with integer operations: the
 // scaling only moves the exponent, so this is exact; v <= 0 (and a subnormal
 // v, whose v 2^E is below 1 for |E| <= 200) gives 0, and results at or above
@@ -91,16 +80,37 @@ __device__ __forceinline__ long long scaled_trunc(double v, int E) {
     return sh >= 0 ? mant << sh : (sh > -53 ? mant >> -sh : 0);
 }
 
+// The weights of up to 32 complex64 amplitudes, summed: with the two squares'
+// sum s and the rest t as above, 0 <= s <= 2^46 and |t| < 2^23, so s = 2^23 h + l
+// with integer h and trunc(l) from additions of 2^23 rounded towards zero (their
+// low mantissa bits are the truncated value), and the halves sum in 32 bits.
+// About 25 FP32 instructions an amplitude, no 64-bit shifts and no conversions.
+struct WeightSum {
+    uint32_t hi = 0, lo = 0;
+    __device__ __forceinline__ void add(float2 z, float sc) {
+        const float re = __fmul_rn(z.x, sc), im = __fmul_rn(z.y, sc);
+        const float pr = __fmul_rn(re, re), er = __fmaf_rn(re, re, -pr);
+        const float pi = __fmul_rn(im, im), ei = __fmaf_rn(im, im, -pi);
+        float s, e;
+        df_two_sum(pr, pi, s, e);
+        const float t = __fadd_rn(__fadd_rn(e, er), ei);
+        constexpr float M = 8388608.f;  // 2^23
+        const float a = __fadd_rz(__fmul_rn(s, 1.f / M), M);
+        const float b = __fadd_rz(__fmaf_rn(-M, __fsub_rn(a, M), s), M);
+        const uint32_t c = __float_as_uint(__fadd_rz(fabsf(t), M)) - 0x4B000000u;
+        hi += __float_as_uint(a) - 0x4B000000u;
+        lo += __float_as_uint(b) - 0x4B000000u;
+        lo += t < 0.f ? 0u - c : c;
+    }
+    // hi <= 32 (2^23 + 1), |lo| < 32 2^24
+    __device__ __forceinline__ long long total() const { return ((long long)hi << 23) + (long long)(int32_t)lo; }
+};
 __device__ __forceinline__ long long weight(float2 z, int E) {
-    const float sc = pow2f(E / 2);
-    const float re = __fmul_rn(z.x, sc), im = __fmul_rn(z.y, sc);
-    const float pr = __fmul_rn(re, re), er = __fmaf_rn(re, re, -pr);
-    const float pi = __fmul_rn(im, im), ei = __fmaf_rn(im, im, -pi);
-    float s, e;
-    df_two_sum(pr, pi, s, e);
-    const float t = __fadd_rn(__fadd_rn(e, er), ei);
-    return trunc_ll(s) + trunc_ll(t);
+    WeightSum w;
+    w.add(z, pow2f(E / 2));
+    return w.total();
 }
+
 __device__ __forceinline__ long long weight(double2 z, int E) {
     return scaled_trunc(z.x * z.x + z.y * z.y, E);
 }
@@ -122,11 +132,15 @@ __device__ __forceinline__ int scale_exp(float m) {
 // coalesced 16-byte loads, pair j of entry e at float4 slot
 // 16 e + ((j + e) & 15): the loads' and the entry reads' quarter-warps hit
 // eight distinct bank quads.
+// Bound by the read of the states now (256 x n = 19, 1.07 GB: about 0.22 ms, 4.9
+// TB/s); each thread keeps its entry in registers between the maximum and the
+// weights, which take 25 instead of about 45 instructions an amplitude.
 constexpr int STAGE_PAIRS = 1 << (GROUP_BITS + ENTRY_BITS - 1);
 constexpr size_t STAGE_BYTES = sizeof(float4) * STAGE_PAIRS;
 template <typename V, bool STAGED>
-__global__ void __launch_bounds__(GROUP) entry_scan_kernel(const V *states, int ns, long long *Q, int *Eg,
-                                                           double *G) {
+__global__ void __launch_bounds__(GROUP, STAGED ? 3 : 1) entry_scan_kernel(const V *states, int ns, long long *Q,
+                                                                           int *Eg, double *G) {
+    pdl_wait();
     __shared__ long long wsum[GROUP / 32];
     __shared__ unsigned int smax;
     const uint64_t N = 1ull << ns, ne = entry_count(ns), ng = group_count(ns);
@@ -147,8 +161,10 @@ __global__ void __launch_bounds__(GROUP) entry_scan_kernel(const V *states, int 
         const float4 *src = reinterpret_cast<const float4 *>(st + gx0);
         for (uint32_t q = threadIdx.x; q < np; q += GROUP) {
             const uint32_t qe = q >> (ENTRY_BITS - 1), qj = q & 15u;
-            stage_buf[16 * qe + ((qj + qe) & 15u)] = src[q];
+            cp_async16(stage_buf + 16 * qe + ((qj + qe) & 15u), src + q);
         }
+        cp_async_commit();
+        cp_async_wait_all();
         stage = stage_buf;
     }
     // amplitude i (< cnt) of this thread's entry
@@ -161,13 +177,38 @@ __global__ void __launch_bounds__(GROUP) entry_scan_kernel(const V *states, int 
         }
     };
     __syncthreads();  // staged tile and smax
-    float m = 0.f;
-    for (uint32_t i = 0; i < cnt; ++i) m = fmaxf(m, prob_f(amp(i)));
-    atomicMax(&smax, __float_as_uint(m));  // nonnegative floats order as their bits
-    __syncthreads();
-    const int E = scale_exp(__uint_as_float(smax));
     long long wv = 0;
-    for (uint32_t i = 0; i < cnt; ++i) wv += weight(amp(i), E);
+    int E;
+    if (STAGED && ((uint64_t)(blockIdx.x + 1) << (GROUP_BITS + ENTRY_BITS)) <= N) {  // a whole group: entries in registers
+        if constexpr (STAGED) {
+            float4 w[16];
+            float m = 0.f;
+#pragma unroll
+            for (uint32_t j = 0; j < 16; ++j) {
+                w[j] = stage[16 * el + ((j + el) & 15u)];
+                m = fmaxf(m, fmaxf(prob_f(make_float2(w[j].x, w[j].y)), prob_f(make_float2(w[j].z, w[j].w))));
+            }
+            const unsigned mb = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));  // nonnegative floats order as their bits
+            if ((el & 31u) == 0) atomicMax(&smax, mb);
+            __syncthreads();
+            E = scale_exp(__uint_as_float(smax));
+            const float sc = pow2f(E / 2);
+            WeightSum ws;
+#pragma unroll
+            for (uint32_t j = 0; j < 16; ++j) {
+                ws.add(make_float2(w[j].x, w[j].y), sc);
+                ws.add(make_float2(w[j].z, w[j].w), sc);
+            }
+            wv = ws.total();
+        }
+    } else {
+        float m = 0.f;
+        for (uint32_t i = 0; i < cnt; ++i) m = fmaxf(m, prob_f(amp(i)));
+        atomicMax(&smax, __float_as_uint(m));
+        __syncthreads();
+        E = scale_exp(__uint_as_float(smax));
+        for (uint32_t i = 0; i < cnt; ++i) wv += weight(amp(i), E);
+    }
     // inclusive scan over the group's 256 entries (exact integer sums)
     const int lane = el & 31, w = el >> 5;
     long long incl = wv;
@@ -195,6 +236,7 @@ __global__ void __launch_bounds__(GROUP) entry_scan_kernel(const V *states, int 
 // offset; the last value of a chunk equals the next chunk's offset, so the
 // result is nondecreasing and rises only where a sum is nonzero.
 __global__ void __launch_bounds__(PREFIX_PT) block_prefix_kernel(double *sums, uint64_t nb) {
+    pdl_wait();
     __shared__ double chunk[PREFIX_PT];
     double *s = sums + (uint64_t)blockIdx.x * nb;
     const uint64_t per = (nb + PREFIX_PT - 1) / PREFIX_PT;
@@ -209,7 +251,8 @@ __global__ void __launch_bounds__(PREFIX_PT) block_prefix_kernel(double *sums, u
     __syncthreads();
     if (threadIdx.x == 0) {
         double acc = 0.0;
-        for (int t = 0; t < PREFIX_PT; ++t) {
+        const int used = (int)((nb + per - 1) / per);  // the other chunks are empty
+        for (int t = 0; t < used; ++t) {
             const double v = chunk[t];
             chunk[t] = acc;
             acc = acc + v;
@@ -224,41 +267,75 @@ __global__ void __launch_bounds__(PREFIX_PT) block_prefix_kernel(double *sums, u
 // which keeps the group search off the FP64 pipe.
 __device__ __forceinline__ long long ord(double v) { return __double_as_longlong(v); }
 
+// A draw is the work of four lanes of a warp (a quad; all 32 lanes call these
+// together).  The four flags of this lane's quad, in bits 0..3:
+__device__ __forceinline__ unsigned quad_ballot(bool p) {
+    return (__ballot_sync(0xFFFFFFFFu, p) >> (threadIdx.x & 28u)) & 15u;
+}
+
 // Smallest i in [0, len) with key(A[i]) > kb (A nondecreasing, the last one
-// qualifies), or >= kb when `ge`; a 32-way search by the whole warp
-// (len < 2^31: at most 2^19 groups, 256 entries).
+// qualifies), or >= kb when `ge`: a 4-way search per quad (len < 2^31: at most
+// 2^19 groups, 256 entries).
 template <typename T, typename K>
-__device__ __forceinline__ uint32_t warp_search(const T *A, uint32_t len, long long kb, bool ge, K key) {
-    const uint32_t lane = threadIdx.x & 31;
+__device__ __forceinline__ uint32_t quad_search(const T *A, uint32_t len, long long kb, bool ge, K key) {
+    const uint32_t q = threadIdx.x & 3;
     uint32_t lo = 0, hi = len;  // the answer is in [lo, hi)
-    while (hi - lo > 1) {
-        const uint32_t stride = (hi - lo + 31) / 32;
-        uint32_t i = lo + (lane + 1) * stride - 1;
+    while (__any_sync(0xFFFFFFFFu, hi - lo > 1)) {
+        const uint32_t stride = (hi - lo + 3) / 4;
+        uint32_t i = lo + (q + 1) * stride - 1;
         if (i > hi - 1) i = hi - 1;
         const long long v = key(A[i]);
-        const unsigned ok = __ballot_sync(0xFFFFFFFFu, ge ? v >= kb : v > kb);
-        const uint32_t f = (uint32_t)(__ffs(ok) - 1);  // A[hi - 1] qualifies, so ok != 0
-        const uint32_t nlo = lo + f * stride;
+        const unsigned ok = quad_ballot(ge ? v >= kb : v > kb);
+        const uint32_t f = ok ? (uint32_t)(__ffs(ok) - 1) : 3u;  // A[hi - 1] qualifies (unless a sum is NaN)
+        const uint32_t nlo = lo + f * stride < hi ? lo + f * stride : hi - 1;
         hi = nlo + stride < hi ? nlo + stride : hi;
         lo = nlo;
     }
     return lo;
 }
 
-// One warp per draw j of instance blockIdx.y: x_j = min { x : F(x) > t } with
+// The eight amplitudes from x on (those at or past N are zero).
+__device__ __forceinline__ void load8(float2 (&z)[8], const float2 *st, uint64_t x, uint64_t N, bool aligned) {
+    if (aligned && x + 8 <= N) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 w = reinterpret_cast<const float4 *>(st + x)[i];
+            z[2 * i] = make_float2(w.x, w.y);
+            z[2 * i + 1] = make_float2(w.z, w.w);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z[i] = x + i < N ? st[x + i] : make_float2(0.f, 0.f);
+    }
+}
+__device__ __forceinline__ void load8(double2 (&z)[8], const double2 *st, uint64_t x, uint64_t N, bool) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) z[i] = x + i < N ? st[x + i] : make_double2(0.0, 0.0);
+}
+
+// Four lanes per draw j of instance blockIdx.y: x_j = min { x : F(x) > t } with
 // t = u_j F_total.  The group comes from the FP64 prefix P; within it the
 // remainder becomes the group's integer units and the rest is exact: the
-// entry from Q, then the first amplitude whose running weight passes it.
-// When t is at F_total, or the remainder at or past the group's integer total
-// (the FP64 group totals are rounded), the last x of nonzero weight of the
-// group is taken; a state of norm zero draws 0.
+// entry from Q, then the first amplitude whose running weight passes it (eight
+// amplitudes per lane).  When t is at F_total, or the remainder at or past the
+// group's integer total (the FP64 group totals are rounded), the last x of
+// nonzero weight of the group is taken; a state of norm zero draws 0.
+//
+// Bound by integer and FP32 issue.  A warp per draw (32-way searches, one
+// amplitude per lane) spent about 430 warp instructions on each, most of them
+// the same in every lane; a quad spends about 60, a lone thread would spend 40
+// but reads its entry's 256 bytes through 16 uncoalesced loads.  Running times of
+// 256 x n = 19 complex64 states, 2^20 draws, with the entry scan: 0.99 -> 0.41 ms
+// a call; 2^22 draws from one n = 26 state 2.38 -> 0.86 ms.
 template <typename V>
-__global__ void __launch_bounds__(DRAW_WARPS * 32) draw_kernel(const V *states, int ns, int z2, const long long *Q,
-                                                                 const int *Eg, const double *P, int k,
-                                                                 const double *u, uint64_t *xs) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t j = (uint64_t)blockIdx.x * DRAW_WARPS + (threadIdx.x >> 5);
-    if (j >= (uint64_t)k) return;  // whole warps leave together
+__global__ void __launch_bounds__(DRAW_PT) draw_kernel(const V *states, int ns, int z2, const long long *Q,
+                                                       const int *Eg, const double *P, int k, const double *u,
+                                                       uint64_t *xs) {
+    pdl_wait();
+    const uint64_t j0 = ((uint64_t)blockIdx.x * DRAW_PT + threadIdx.x) >> 2;
+    const bool live = j0 < (uint64_t)k;  // the others draw along, for the warp's votes
+    const uint64_t j = live ? j0 : (uint64_t)k - 1;
+    const uint32_t q = threadIdx.x & 3;
     const uint64_t inst = blockIdx.y;
     const uint64_t N = 1ull << ns, ne = entry_count(ns), ng = group_count(ns);
     const V *st = states + (inst << ns);
@@ -279,7 +356,7 @@ __global__ void __launch_bounds__(DRAW_WARPS * 32) draw_kernel(const V *states, 
     // group (t and the sums are >= +0)
     bool edge = ord(t) >= ord(total);
     auto dkey = [](double v) { return ord(v); };
-    const uint64_t g = warp_search(Pi, (uint32_t)ng, ord(edge ? total : t), edge, dkey);
+    const uint64_t g = quad_search(Pi, (uint32_t)ng, ord(edge ? total : t), edge, dkey);
     const int E = Eg[inst * ng + g];
     // the remainder in the group's integer units
     const uint64_t e0 = g << GROUP_BITS;
@@ -292,22 +369,38 @@ __global__ void __launch_bounds__(DRAW_WARPS * 32) draw_kernel(const V *states, 
         edge = R >= Ig;
     }
     auto ikey = [](long long v) { return v; };
-    const uint64_t e = warp_search(Qg, (uint32_t)glen, edge ? Ig : R, edge, ikey);
+    const uint64_t e = quad_search(Qg, (uint32_t)glen, edge ? Ig : R, edge, ikey);
     R -= e > 0 ? Qg[e - 1] : 0;
     // amplitude within the entry: exact integer running weights
-    const uint64_t x = ((e0 + e) << ENTRY_BITS) + (uint64_t)lane;
-    const long long wv = x < N ? weight(st[x], E) : 0;
-    long long incl = wv;
+    const uint64_t x0 = (e0 + e) << ENTRY_BITS;
+    V z[8];
+    load8(z, st, x0 + 8 * q, N, (reinterpret_cast<uintptr_t>(states) & 15u) == 0);
+    long long w[8], sum = 0;
+    int last = -1;  // last amplitude of this lane with a weight
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
+    for (int i = 0; i < 8; ++i) {
+        w[i] = weight(z[i], E);
+        sum += w[i];
+        if (w[i] > 0) last = i;
     }
-    const unsigned hit = __ballot_sync(0xFFFFFFFFu, !edge && incl > R);
-    const unsigned nz = __ballot_sync(0xFFFFFFFFu, wv > 0);
-    const int pick = hit ? __ffs(hit) - 1 : (nz ? 31 - __clz(nz) : 0);
-    if (lane == 0) {
-        const uint64_t found = ((e0 + e) << ENTRY_BITS) + (uint64_t)pick;
+    long long run = sum;  // inclusive over the quad, then this lane's start
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const long long y = __shfl_up_sync(0xFFFFFFFFu, run, o, 4);
+        if ((int)q >= o) run += y;
+    }
+    const bool has = !edge && run > R;  // the quad's first such lane holds the draw
+    run -= sum;
+    int pick = 0;  // first amplitude whose running weight passes R: those before do not
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+        run += w[i];
+        pick += run <= R ? 1 : 0;
+    }
+    const unsigned hit = quad_ballot(has), nz = quad_ballot(last >= 0);
+    const uint32_t lane = hit ? (uint32_t)(__ffs(hit) - 1) : (nz ? 31u - (uint32_t)__clz((int)nz) : 0u);
+    if (live && q == lane) {
+        const uint64_t found = x0 + 8 * q + (uint64_t)(hit ? pick : (last >= 0 ? last : 0));
         const uint64_t full = (1ull << (ns + (z2 ? 1 : 0))) - 1ull;
         xs[inst * (uint64_t)k + j] = flip ? (~found & full) : found;
     }
@@ -317,6 +410,7 @@ __global__ void __launch_bounds__(DRAW_WARPS * 32) draw_kernel(const V *states, 
 // With a half table (z2) an x with bit n-1 set is looked up as its complement,
 // C(not x) = C(x).
 __global__ void first_hit_kernel(const uint8_t *costs, int nc, int z2, int k, const uint64_t *xs, int *first) {
+    pdl_wait();
     const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t inst = blockIdx.y;
     if (j >= (uint64_t)k) return;
@@ -355,7 +449,8 @@ static int sample_impl(int batch, int n, const uint8_t *d_costs, const void *d_s
     double *d_pre = reinterpret_cast<double *>(dev + qb + eb);
     uint64_t *xs = d_x ? d_x : reinterpret_cast<uint64_t *>(dev + pre);
     int *d_first = reinterpret_cast<int *>(dev + pre + xb);
-    const dim3 draw_grid((unsigned)((k + DRAW_WARPS - 1) / DRAW_WARPS), batch);
+    const dim3 draw_grid((unsigned)(((uint64_t)k * 4 + DRAW_PT - 1) / DRAW_PT), batch);
+    if (running_time) QAOA_CUDA_TRY(cudaMemsetAsync(d_first, 0x7F, fb, stream));  // 0x7F7F7F7F > any draw index
     profile_before(K_SAMPLE, stream);
     if (dtype == QAOA_C64) {
         const float2 *st = reinterpret_cast<const float2 *>(d_states);
@@ -364,26 +459,23 @@ static int sample_impl(int batch, int n, const uint8_t *d_costs, const void *d_s
             const cudaError_t attr = cudaFuncSetAttribute(
                 entry_scan_kernel<float2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STAGE_BYTES);
             if (attr != cudaSuccess) return cuda_error(attr, "entry scan shared memory");
-            entry_scan_kernel<float2, true><<<dim3((unsigned)ng, batch), GROUP, STAGE_BYTES, stream>>>(st, ns, d_q,
-                                                                                                      d_e, d_pre);
+            launch_pdl(entry_scan_kernel<float2, true>, dim3((unsigned)ng, batch), dim3(GROUP), STAGE_BYTES, stream, st, ns,
+                       d_q, d_e, d_pre);
         } else {
-            entry_scan_kernel<float2, false><<<dim3((unsigned)ng, batch), GROUP, 0, stream>>>(st, ns, d_q, d_e, d_pre);
+            launch_pdl(entry_scan_kernel<float2, false>, dim3((unsigned)ng, batch), dim3(GROUP), 0, stream, st, ns, d_q, d_e, d_pre);
         }
-        block_prefix_kernel<<<batch, PREFIX_PT, 0, stream>>>(d_pre, ng);
-        draw_kernel<float2><<<draw_grid, DRAW_WARPS * 32, 0, stream>>>(st, ns, z2 ? 1 : 0, d_q, d_e, d_pre, k, d_u,
-                                                                       xs);
+        launch_pdl(block_prefix_kernel, dim3(batch), dim3(PREFIX_PT), 0, stream, d_pre, ng);
+        launch_pdl(draw_kernel<float2>, draw_grid, dim3(DRAW_PT), 0, stream, st, ns, z2 ? 1 : 0, d_q, d_e, d_pre, k, d_u, xs);
     } else {
         const double2 *st = reinterpret_cast<const double2 *>(d_states);
-        entry_scan_kernel<double2, false><<<dim3((unsigned)ng, batch), GROUP, 0, stream>>>(st, ns, d_q, d_e, d_pre);
-        block_prefix_kernel<<<batch, PREFIX_PT, 0, stream>>>(d_pre, ng);
-        draw_kernel<double2><<<draw_grid, DRAW_WARPS * 32, 0, stream>>>(st, ns, z2 ? 1 : 0, d_q, d_e, d_pre, k, d_u,
-                                                                        xs);
+        launch_pdl(entry_scan_kernel<double2, false>, dim3((unsigned)ng, batch), dim3(GROUP), 0, stream, st, ns, d_q, d_e, d_pre);
+        launch_pdl(block_prefix_kernel, dim3(batch), dim3(PREFIX_PT), 0, stream, d_pre, ng);
+        launch_pdl(draw_kernel<double2>, draw_grid, dim3(DRAW_PT), 0, stream, st, ns, z2 ? 1 : 0, d_q, d_e, d_pre, k, d_u, xs);
     }
     rc = profile_after(K_SAMPLE, stream);
     if (rc || !running_time) return rc;
-    QAOA_CUDA_TRY(cudaMemsetAsync(d_first, 0x7F, fb, stream));  // 0x7F7F7F7F > any draw index
-    first_hit_kernel<<<dim3((unsigned)((k + 255) / 256), batch), 256, 0, stream>>>(d_costs, ns, z2 ? 1 : 0, k, xs,
-                                                                                    d_first);
+    launch_pdl(first_hit_kernel, dim3((unsigned)((k + 255) / 256), batch), dim3(256), 0, stream, d_costs, ns, z2 ? 1 : 0, k,
+               (const uint64_t *)xs, d_first);
     QAOA_CUDA_TRY(cudaGetLastError());
     int *h = reinterpret_cast<int *>(sc->host);
     QAOA_CUDA_TRY(cudaMemcpyAsync(h, d_first, fb, cudaMemcpyDeviceToHost, stream));
