@@ -167,13 +167,6 @@ __device__ __forceinline__ void rounds_down(typename G::V *v, typename G::V *til
 // inside one instance fit in 32 bits (n <= 32).
 // sc: the tile's cost bytes in shared memory, indexed by tile element (by
 // landing position when Z2).
-// |v|^2 and a zero amplitude for each arithmetic (double-float: in FP64).
-__device__ __forceinline__ float amp_prob(const float2 &v) { return v.x * v.x + v.y * v.y; }
-__device__ __forceinline__ double amp_prob(const double2 &v) { return v.x * v.x + v.y * v.y; }
-__device__ __forceinline__ double amp_prob(const float4 &v) {
-    const double re = (double)v.x + (double)v.y, im = (double)v.z + (double)v.w;
-    return re * re + im * im;
-}
 template <typename V>
 __device__ __forceinline__ V zero_amp() {
     V z;
@@ -746,7 +739,7 @@ static void fill_table(PhaseTab<R, MAX_TABLE> *tab, const EvolveReq &r, int l, i
     const LayerCoef k = r.p > 0 ? layer_coef(r.beta[l], sign, arith_of(r.dtype, r.flags)) : LayerCoef{1.0, 1.0, 0.0, true};
     double scale = layer_scale(k, r.n);
     if (l == 0) scale *= std::pow(2.0, -0.5 * r.n);
-    phase_table(r.p > 0 ? r.gamma[l] : 0.0, scale, r.m, re.data(), im.data());
+    phase_table(r.p > 0 ? r.gamma[l] : 0.0, scale, r.m, arith_of(r.dtype, r.flags), re.data(), im.data());
     for (int c = 0; c <= r.m; ++c) tab->t[c] = amp_from(&tab->t[c], re[c], im[c]);
 }
 
@@ -963,6 +956,17 @@ static int evolve_common(int batch, int n, const uint8_t *d_cost, int m, int p, 
         return QAOA_OK;
     }
     if (n <= small_n_limit(dtype)) return set_error(QAOA_ERANGE, "n=%d too small for the pass path", n);
+    if (!adj) {  // a few mid-sized instances: one cooperative launch
+        bool taken = false;
+        std::vector<double> h(want ? 2 * (size_t)batch : 0);
+        rc = evolve_mid(r, stream, want ? h.data() : nullptr, &taken);
+        if (rc) return rc;
+        for (int b = 0; taken && want && b < batch; ++b) {
+            if (p_succ) p_succ[b] = scale * h[2 * b];
+            if (norm) norm[b] = scale * h[2 * b + 1];
+        }
+        if (taken) return QAOA_OK;
+    }
     // a full table's evolution works on half of the amplitudes when the table is
     // flip-symmetric (checked on the device, instance by instance)
     const int gx = pass_grid_x(dtype, p > 0 || z2 ? n - 1 : n, batch);

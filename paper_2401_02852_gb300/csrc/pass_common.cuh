@@ -418,6 +418,13 @@ __device__ __forceinline__ void issue_tile(const typename G::V *st, const uint8_
     }
 }
 
+// |v|^2 for each arithmetic (double-float: in FP64).
+__device__ __forceinline__ float amp_prob(const float2 &v) { return v.x * v.x + v.y * v.y; }
+__device__ __forceinline__ double amp_prob(const double2 &v) { return v.x * v.x + v.y * v.y; }
+__device__ __forceinline__ double amp_prob(const float4 &v) {
+    const double re = (double)v.x + (double)v.y, im = (double)v.z + (double)v.w;
+    return re * re + im * im;
+}
 // Halved state (low pass): tile element u with bit T-1 set is the mirror
 // 2^(n-1) - 1 - x of the element x = u with that bit clear; its data and cost
 // bytes land in reverse memory order at position 2^T - 1 - (u mod 2^(T-1)).

@@ -40,11 +40,15 @@ struct Scratch {
     size_t dev_bytes = 0;
     void *host = nullptr;  // pinned host bytes
     size_t host_bytes = 0;
+    unsigned *bars = nullptr;  // grid-barrier words, left fit for the next launch by each
+    size_t n_bars = 0;
 };
 // Returns scratch for `stream` on the current device with at least the given
 // capacities (device, pinned host).  Not thread-safe per stream: one caller
 // thread per stream at a time, as for any CUDA stream.
 int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratch **out);
+// The stream's barrier words (at least `count`; kernels leave them as found).
+int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out);
 // Kernel attributes (the dynamic shared-memory limit) belong to a device:
 // the current device's ordinal for per-device set-up state, or -1 with the
 // error recorded when it is out of [0, MAX_DEVICES).
@@ -68,6 +72,7 @@ enum KernelKind {
     K_FLIP_CHECK,
     K_MIRROR,
     K_ENCODE,
+    K_MID,
     K_NUM_KINDS
 };
 // Call before / after a launch on `stream`.  `after` checks the launch status.
@@ -178,8 +183,12 @@ inline int arith_of(int dtype, int flags) {
 }
 
 // Phase table of one layer: T[c] = scale * exp(-i gamma c), c = 0..m (FP64 on
-// the host; cast to the state's element type by the caller).
-void phase_table(double gamma, double scale, int m, double *re, double *im);
+// the host; cast to the state's element type by the caller).  For complex64 and
+// double-float tables (ARITH_F32, ARITH_DF) only every eighth entry is evaluated,
+// the others are its products with exp(-i gamma b), b < 8: a few units of 2^-53,
+// far below those types' last places, at a fifth of the time (a host that fills
+// 10 layers of 129 entries ahead of one launch waits 30 us for them otherwise).
+void phase_table(double gamma, double scale, int m, int arith, double *re, double *im);
 
 // Largest cost a phase table indexes.  The cost table is uint8, so
 // C(x) <= 255 whatever m is: a table holds entries 0..table_top(m).
@@ -267,6 +276,11 @@ int launch_small_batch(int dtype, int n_jobs, const SmallJob *d_jobs, const void
 // the stream when it staged them or r.d_result is set.
 size_t small_stage_bytes(int dtype, int m, int p);
 int evolve_small(const EvolveReq &r, void *h_stage, void *d_stage, cudaStream_t stream);
+// Whole evolutions (p >= 1, no adjoint seed) of as many mid-sized instances as
+// the device holds at once, in one cooperative launch: *taken is false (and
+// nothing was done) when r is not such a request.  With h_result (host [batch][2])
+// waits for the results.
+int evolve_mid(const EvolveReq &r, cudaStream_t stream, double *h_result, bool *taken);
 // Gradients for n at most small_n_limit (through the stream's scratch).  Waits
 // for the stream.
 int grad_small(int batch, int n, const uint8_t *cost, int m, int p, const double *gamma, const double *beta, int dtype,

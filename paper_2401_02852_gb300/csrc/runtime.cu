@@ -108,6 +108,24 @@ int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratc
     return QAOA_OK;
 }
 
+int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out) {
+    if (s->n_bars < count) {
+        QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
+        if (s->bars) cudaFree(s->bars);
+        s->bars = nullptr;
+        s->n_bars = 0;
+        const size_t want = count < 1024 ? 1024 : count;
+        if (cudaMalloc((void **)&s->bars, want * sizeof(unsigned)) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(QAOA_ENOMEM, "scratch: %zu barrier words", want);
+        }
+        QAOA_CUDA_TRY(cudaMemsetAsync(s->bars, 0, want * sizeof(unsigned), stream));
+        s->n_bars = want;
+    }
+    *out = s->bars;
+    return QAOA_OK;
+}
+
 static int release_all_scratch() {
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     int cur = 0;
@@ -117,6 +135,7 @@ static int release_all_scratch() {
         cudaDeviceSynchronize();
         if (kv.second.dev) cudaFree(kv.second.dev);
         if (kv.second.host) cudaFreeHost(kv.second.host);
+        if (kv.second.bars) cudaFree(kv.second.bars);
     }
     g_scratch.clear();
     cudaSetDevice(cur);
@@ -137,7 +156,7 @@ static thread_local cudaEvent_t t_pending = nullptr;
 
 static const char *k_names[K_NUM_KINDS] = {
     "cost_table", "pass_low", "pass_high", "small_n", "reduce",
-    "success_prob", "adjoint_low", "adjoint_high", "adjoint_seed", "serve_small", "sample", "flip_check", "mirror", "encode"};
+    "success_prob", "adjoint_low", "adjoint_high", "adjoint_seed", "serve_small", "sample", "flip_check", "mirror", "encode", "mid"};
 
 static cudaEvent_t take_event() {
     std::lock_guard<std::mutex> lk(g_prof_mu);
@@ -332,7 +351,22 @@ LayerCoef layer_coef(double beta, int sign, int arith) {
     return k;
 }
 
-void phase_table(double gamma, double scale, int m, double *re, double *im) {
+void phase_table(double gamma, double scale, int m, int arith, double *re, double *im) {
+    if (arith != ARITH_F64) {
+        constexpr int S = 8;
+        double br[S], bi[S];
+        for (int b = 1; b < S; ++b) br[b] = std::cos(gamma * (double)b), bi[b] = -std::sin(gamma * (double)b);
+        for (int c = 0; c <= m; c += S) {
+            const double x = scale * std::cos(gamma * (double)c), y = -scale * std::sin(gamma * (double)c);
+            re[c] = x;
+            im[c] = y;
+            for (int b = 1; b < S && c + b <= m; ++b) {
+                re[c + b] = x * br[b] - y * bi[b];
+                im[c + b] = x * bi[b] + y * br[b];
+            }
+        }
+        return;
+    }
     for (int c = 0; c <= m; ++c) {
         re[c] = scale * std::cos(gamma * (double)c);
         im[c] = -scale * std::sin(gamma * (double)c);

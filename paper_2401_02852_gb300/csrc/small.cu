@@ -34,6 +34,7 @@
 #include <mutex>
 #include <vector>
 
+#include "orbits.cuh"
 #include "pass_common.cuh"
 #include "qaoa_internal.cuh"
 
@@ -41,33 +42,9 @@ namespace qaoa {
 
 namespace cg = cooperative_groups;
 
-// One layer's coefficients, 32 bytes in complex128 and double-float.
-template <typename R>
-struct SmallCoef {
-    R A, B;
-    int unit_a;
-    double sigma2;
-};
-static_assert(sizeof(SmallCoef<double>) == 32 && sizeof(SmallCoef<dfloat>) == 32, "one stride for complex128");
-
-// Bytes of p layers' tables, up to the coefficients behind them.
-__host__ __device__ inline size_t small_table_bytes(size_t entry, int p, int m) {
-    return (entry * (size_t)p * (size_t)(m + 1) + 15) & ~(size_t)15;
-}
-
 constexpr int SMALL_PT = 256;     // threads of a CTA that is alone
 constexpr int SMALL_PT_CL = 128;  // ... in a cluster
 constexpr int SMALL_SYM_N = 6;    // smallest n held as a half
-
-template <typename V>
-__device__ __forceinline__ uint32_t swz(uint32_t i) {
-    return sizeof(V) == 8 ? i ^ ((i >> 4) & 15u) : i ^ ((i >> 3) & 7u) ^ ((i >> 6) & 7u);
-}
-
-// An amplitude in FP64.
-__device__ __forceinline__ double2 amp_f64(float2 v) { return make_double2(v.x, v.y); }
-__device__ __forceinline__ double2 amp_f64(double2 v) { return v; }
-__device__ __forceinline__ double2 amp_f64(float4 v) { return make_double2((double)v.x + v.y, (double)v.z + v.w); }
 
 // Where a CTA's part of the state lies and how its orbits are addressed.
 template <typename V, int CB>
@@ -94,52 +71,6 @@ struct Part {
         else
             return cg::this_cluster().map_shared_rank(s, r);
     }
-};
-
-// Calls f(byte offsets of the 2^K members in the state, representative) for this
-// thread's orbits of a local round: acting bits [j, j + K), the lowest of them
-// standing for the complement when `mir` (CB = 0).
-template <typename V, int K, int CB, class F>
-__device__ __forceinline__ void local_orbits(const Part<V, CB> &pt, int j, bool mir, const F &f) {
-    const uint32_t L = 1u << pt.lb;
-    uint32_t m[K];
-#pragma unroll
-    for (int q = 0; q < K; ++q) m[q] = swz<V>(q == 0 && mir ? L - 1u : 1u << (j + q)) * (uint32_t)sizeof(V);
-    for (uint32_t g = threadIdx.x; g < L >> K; g += blockDim.x) {
-        const uint32_t z0 = ((g >> j) << (j + K)) | (g & ((1u << j) - 1u));
-        uint32_t off[1 << K];
-        off[0] = swz<V>(z0) * (uint32_t)sizeof(V);
-#pragma unroll
-        for (int q = 0; q < K; ++q)
-#pragma unroll
-            for (int r = 0; r < (1 << q); ++r) off[r | (1 << q)] = off[r] ^ m[q];
-        f(off, z0);
-    }
-}
-
-template <typename V>
-__device__ __forceinline__ V &at(V *s, uint32_t off) {
-    return *reinterpret_cast<V *>(reinterpret_cast<char *>(s) + off);
-}
-
-// The costs of 2^K consecutive amplitudes (sc aligned to them).
-template <int K>
-struct CostBytes {
-    uint32_t w[K > 2 ? 1 << (K - 2) : 1];
-    __device__ __forceinline__ explicit CostBytes(const uint8_t *sc) {
-        if constexpr (K == 1) {
-            w[0] = *reinterpret_cast<const uint16_t *>(sc);
-        } else if constexpr (K == 2) {
-            w[0] = *reinterpret_cast<const uint32_t *>(sc);
-        } else if constexpr (K == 3) {
-            const uint2 t = *reinterpret_cast<const uint2 *>(sc);
-            w[0] = t.x, w[1] = t.y;
-        } else {
-            const uint4 t = *reinterpret_cast<const uint4 *>(sc);
-            w[0] = t.x, w[1] = t.y, w[2] = t.z, w[3] = t.w;
-        }
-    }
-    __device__ __forceinline__ uint32_t operator[](int r) const { return (w[r >> 2] >> (8 * (r & 3))) & 0xFFu; }
 };
 
 // The same for remote round i: generators 2 i and 2 i + 1 of [the complement
@@ -215,16 +146,6 @@ __device__ __forceinline__ void barrier(bool wide) {
     __syncthreads();
 }
 
-// K butterflies on an orbit.
-template <bool UA, int K, typename V, typename R>
-__device__ __forceinline__ void orbit_bfly(V *v, R A, R B) {
-#pragma unroll
-    for (int q = 0; q < K; ++q)
-#pragma unroll
-        for (int i = 0; i < (1 << K); ++i)
-            if (!(i & (1 << q))) bfly<UA>(v[i], v[i | (1 << q)], A, B);
-}
-
 // The inverse butterflies with B = 1, (a, b) <- (A a - i b, A b - i a).
 template <int K, typename V, typename R>
 __device__ __forceinline__ void inv_orbit(V *v, R A) {
@@ -283,29 +204,6 @@ __device__ __forceinline__ void load_costs(uint8_t *sc, const uint8_t *cost, uin
     }
 }
 
-// The phase table of one layer, fetched ahead into registers (entries tid + k
-// blockDim) and put into shared memory later; entries above m are zero.
-constexpr int TAB_REGS = MAX_TABLE / 128;  // at least 128 threads
-template <typename V>
-struct TabAhead {
-    V e[TAB_REGS];
-    __device__ __forceinline__ void fetch(const V *tb, int m) {
-#pragma unroll
-        for (int k = 0; k < TAB_REGS; ++k) {
-            const int c = (int)(threadIdx.x + k * blockDim.x);
-            memset(&e[k], 0, sizeof(V));
-            if (c < MAX_TABLE && c <= m) e[k] = tb[c];
-        }
-    }
-    __device__ __forceinline__ void put(V *stab) const {
-#pragma unroll
-        for (int k = 0; k < TAB_REGS; ++k) {
-            const int c = (int)(threadIdx.x + k * blockDim.x);
-            if (c < MAX_TABLE) stab[c] = e[k];
-        }
-    }
-};
-
 // p >= 1 layers forward from |+>; s holds the CTA's part afterwards.  tb0, cf0:
 // the layers' tables [p][m + 1] and coefficients [p].  On return the last
 // layer's table is in stab + ((p - 1) & 1) MAX_TABLE and the state is visible to
@@ -328,7 +226,7 @@ __device__ __forceinline__ void forward_layers(const Part<V, CB> &pt, V *s, V *s
         }
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
             constexpr int K = decltype(kc)::value;
-            local_orbits<V, K, CB>(pt, j, mir, [&](const uint32_t(&off)[1 << K], uint32_t z0) {
+            orbits<V, K>(pt.lb, j, mir, [&](const uint32_t(&off)[1 << K], uint32_t z0) {
                 V v[1 << K];
                 if (first) {  // j = 0: the members are consecutive
                     const CostBytes<K> c(sc + z0);
@@ -578,7 +476,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
             constexpr int K = decltype(kc)::value;
             R t = 0, g0 = 0, g1 = 0;
-            local_orbits<V, K, CB>(pt, j, mir, [&](const uint32_t(&off)[1 << K], uint32_t z0) {
+            orbits<V, K>(pt.lb, j, mir, [&](const uint32_t(&off)[1 << K], uint32_t z0) {
                 V v[1 << K], u[1 << K];
 #pragma unroll
                 for (int r = 0; r < (1 << K); ++r) v[r] = at(s, off[r]);
@@ -790,7 +688,7 @@ static void fill_layer(int n, int m, double gamma, double beta, bool layer, bool
     double scale = layer_scale(k, n);
     if (first) scale *= std::pow(2.0, -0.5 * n);
     double re[MAX_TABLE], im[MAX_TABLE];
-    phase_table(layer ? gamma : 0.0, scale, m, re, im);
+    phase_table(layer ? gamma : 0.0, scale, m, arith, re, im);
     V *t = reinterpret_cast<V *>(tab);
     for (int c = 0; c <= m; ++c) {
         if constexpr (std::is_same<R, dfloat>::value) {
