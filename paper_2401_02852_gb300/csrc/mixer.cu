@@ -197,15 +197,30 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
         const uint32_t o = (u & ((1u << ROW) - 1u)) + (u >> ROW) * gstride;
         return (Z2 && mirror) ? -(int64_t)o : (int64_t)o;
     };
-    if (is_df<R>() && RED && reduce) {  // the evolution's last pass: FP64 out
+    if (is_df<R>() && RED && reduce) {
+        // The evolution's last pass: FP64 out, and the sums from the same values.
+        // Bound by the FP64 pipe, so the floats are widened by integer operations
+        // and only solutions add to p_succ: 5 FP64 operations per amplitude instead
+        // of about 11.
         double2 *sd = reinterpret_cast<double2 *>(sp);
+        PairwiseSum<NR, double> nm;
+        double ps = 0.0;
+        const uint32_t tid = threadIdx.x;
+        const uint32_t cb = PADC ? cost_base<Cx<R>, LO>(tid) : 0u;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
             const float4 w = *reinterpret_cast<const float4 *>(&v[r]);
-            const double2 d = make_double2((double)w.x + (double)w.y, (double)w.z + (double)w.w);
+            const double2 d = make_double2(widen(w.x) + widen(w.y), widen(w.z) + widen(w.w));
             sd[off(r)] = d;
             if (mp) reinterpret_cast<double2 *>(mp)[-off(r)] = d;
+            const double pr = d.x * d.x + d.y * d.y;
+            nm.add(r, pr);
+            const uint32_t u = tile_elem<Cx<R>, LO>(tid, r);
+            if (sc[PADC ? cb + Cx<R>::cidx((uint32_t)r << LO) : (Z2 ? land<Cx<R>::T>(u) : u)] == 0) ps += pr;
         }
+        acc[0] += ps;
+        acc[1] += nm.total();
+        return;
     } else if constexpr (is_df<R>()) {  // pairs renormalised between passes
 #pragma unroll
         for (int r = 0; r < NR; ++r) sp[off(r)] = df_renorm(v[r]);
@@ -247,9 +262,9 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
 // copy chunks j < EARLY_ELEMS / (2 PT) (6 of 16): both splits are compile-time.
 // 24 KiB more per CTA (108.5 KiB), still two CTAs per SM.
 constexpr int EARLY_ELEMS = 3072;
-template <typename R, bool LOW, int MODE, int NB>
+template <typename R, bool LOW, int MODE, int NB, int HROW>
 __host__ __device__ constexpr bool early_landing() {
-    return !LOW && MODE == MODE_FUSED && NB == 1 && std::is_same<R, float>::value;
+    return !LOW && MODE == MODE_FUSED && NB == 1 && std::is_same<R, float>::value && HROW < Cx<R>::LOAD;
 }
 
 // NB = 1: one tile buffer per CTA, two CTAs per SM; the next tile's copies
@@ -264,7 +279,11 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half
     using V = typename G::V;
     constexpr int T = G::T, NR = G::NR;
     constexpr int LD = G::LOAD;                // first round's mapping
-    constexpr int LC = LastLO<G, LOW>::value;  // last round's mapping
+    // Rows of 2^LOAD amplitudes and more: every qubit of the group is a register
+    // bit of the load mapping, so the pass needs no exchange; the next tile's
+    // copies start as soon as this one is in registers.
+    constexpr bool TOP = !LOW && HROW >= LD;
+    constexpr int LC = TOP ? LD : LastLO<G, LOW>::value;  // last round's mapping
     const uint32_t tid = threadIdx.x;
     const size_t inst = blockIdx.y;
     V *st = a.state + (inst << a.n);
@@ -308,7 +327,7 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half
     };
     auto tbuf = [&](int b) { return tiles_buf + (size_t)b * G::TILE_ELEMS; };
     auto cbuf = [&](int b) { return scs + (size_t)b * G::CS_BYTES; };
-    constexpr bool EARLY = early_landing<R, LOW, MODE, NB>();
+    constexpr bool EARLY = early_landing<R, LOW, MODE, NB, HROW>();
     constexpr int JE = EARLY_ELEMS / ((16 / (int)sizeof(V)) * G::PT);  // early copy chunks per thread
     constexpr int RE = EARLY_ELEMS >> LD;                              // early load-mapping registers
     static_assert(!EARLY || ((RE << LD) == EARLY_ELEMS && JE * (16 / (int)sizeof(V)) * G::PT == EARLY_ELEMS),
@@ -405,7 +424,19 @@ __device__ __forceinline__ void pass_tiles(const PassArgs<R> &a, const bool half
             else
                 v[r] = (EARLY && r < RE) ? ebuf[u] : tile[u];
         }
-        if (MODE == MODE_FUSED) {
+        using R0 = typename PassRounds<G, LOW>::R0;
+        if constexpr (TOP) {
+            prefetch();
+            mask_butterflies<G, UA1, R0::LO, R0::MASK>(v, active, a.A1, a.B1);
+            if (MODE == MODE_FUSED) {
+#pragma unroll
+                for (int r = 0; r < NR; ++r) v[r] = cmul(v[r], stab[sc[cbl + G::cidx((uint32_t)r << LD)]]);
+                mask_butterflies<G, UA2, R0::LO, R0::MASK>(v, active, a.A2, a.B2);
+            }
+            const uint32_t x0 = base + ld_t;
+            store_tile<R, LD, row, false, RED, true>(v, st + x0, sc, adj ? adj + x0 : nullptr,
+                                                     expand ? st + (2ull * M + 1 - x0) : nullptr, gstride, false, red, acc);
+        } else if (MODE == MODE_FUSED) {
             rounds_up<G, LOW, UA1>(v, tile, active, a.A1, a.B1, early_hook);
             const uint32_t cb = cost_base<G, LC>(tid);
 #pragma unroll
@@ -472,7 +503,7 @@ __global__ void __launch_bounds__(Cx<R>::PT, NB == 3 ? 1 : 2) pass_kernel(const 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *tile = reinterpret_cast<V *>(smem_raw);
     uint8_t *scs = reinterpret_cast<uint8_t *>(tile + (size_t)NB * Cx<R>::TILE_ELEMS);
-    constexpr bool EARLY = early_landing<R, LOW, MODE, NB>();
+    constexpr bool EARLY = early_landing<R, LOW, MODE, NB, HROW>();
     V *ebuf = EARLY ? reinterpret_cast<V *>(scs + (size_t)NCB * Cx<R>::CS_BYTES) : nullptr;
     V *stab = reinterpret_cast<V *>(scs + (size_t)NCB * Cx<R>::CS_BYTES + (EARLY ? EARLY_ELEMS * sizeof(V) : 0));
     if (MODE != MODE_PLAIN) {  // 256 entries at least: any uint8 cost indexes inside the table
@@ -586,6 +617,56 @@ struct HighSet {
     }
 };
 
+// A last group with fewer new qubits than a narrow group holds: instead of the
+// carried bits its tiles take longer rows, 2^HROW amplitudes, so every bit of the
+// group is butterflied (a compile-time mask) and the rows stream better.  It is
+// never the first pass of an evolution.
+template <typename R, int SYM, int HROW>
+struct TailSet {
+    using Full = PhaseTab<R, MAX_TABLE>;
+    using None = PhaseTab<R, 1>;
+    void (*plain[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, false, MODE_PLAIN, false, false, 1, false, HROW, true>,
+                                           pass_kernel<R, SYM, false, MODE_PLAIN, true, false, 1, false, HROW, true>};
+    void (*plain_red[2])(PassArgs<R>, None) = {pass_kernel<R, SYM, false, MODE_PLAIN, false, false, 1, true, HROW, true>,
+                                               pass_kernel<R, SYM, false, MODE_PLAIN, true, false, 1, true, HROW, true>};
+    void (*fused[2][2])(PassArgs<R>, Full) = {
+        {pass_kernel<R, SYM, false, MODE_FUSED, false, false, MAX_TABLE, false, HROW, true>,
+         pass_kernel<R, SYM, false, MODE_FUSED, false, true, MAX_TABLE, false, HROW, true>},
+        {pass_kernel<R, SYM, false, MODE_FUSED, true, false, MAX_TABLE, false, HROW, true>,
+         pass_kernel<R, SYM, false, MODE_FUSED, true, true, MAX_TABLE, false, HROW, true>}};
+    void all(std::vector<KPtr> &ks) const {
+        for (int i = 0; i < 2; ++i) {
+            ks.push_back((KPtr)plain[i]);
+            ks.push_back((KPtr)plain_red[i]);
+            for (int j = 0; j < 2; ++j) ks.push_back((KPtr)fused[i][j]);
+        }
+    }
+};
+
+// Tail sets for rows of HROW .. LAST bits.
+template <typename R, int SYM, int HROW, int LAST>
+struct Tails {
+    TailSet<R, SYM, HROW> set;
+    Tails<R, SYM, HROW + 1, LAST> next;
+    void all(std::vector<KPtr> &ks) const {
+        set.all(ks);
+        next.all(ks);
+    }
+    template <class F>
+    void with(int row, const F &f) const {
+        if (row == HROW)
+            f(set);
+        else
+            next.with(row, f);
+    }
+};
+template <typename R, int SYM, int LAST>
+struct Tails<R, SYM, LAST + 1, LAST> {
+    void all(std::vector<KPtr> &) const {}
+    template <class F>
+    void with(int, const F &) const {}
+};
+
 // The kernels of the low pass (NB: tile buffers per CTA); all butterfly every
 // tile bit, except init0 (p = 0: the initial state alone).
 template <typename R, int SYM, int NB = 1>
@@ -622,8 +703,11 @@ template <typename R, int SYM>
 struct PassKernels {
     using Full = PhaseTab<R, MAX_TABLE>;
     using None = PhaseTab<R, 1>;
-    // high passes with rows of WROW bits (complex64: 32 amplitudes, 256 B);
-    // complex128 has no wide rows and those are the narrow kernels again
+    // complex64 high passes take rows of WROW bits (32 amplitudes, 256 B) where
+    // the plan has them.  Last groups with fewer bits take longer rows (TailSet),
+    // except in FP64, whose pipe bounds its passes either way: those carry the
+    // other bits and butterfly with a runtime mask (high_part).
+    static constexpr bool FP64 = std::is_same<R, double>::value;
     static constexpr int WROW = sizeof(R) == 4 ? HIGH_ROW + 1 : HIGH_ROW;
     LowSet<R, SYM> low;
     // One CTA per SM, three tile buffers: the complex64 low passes of a single
@@ -632,19 +716,19 @@ struct PassKernels {
     // batched low passes all run slower with one CTA per SM.)
     static constexpr bool NB3 = std::is_same<R, float>::value;
     typename std::conditional<NB3, LowSet<R, SYM, 3>, NoLowSet<R>>::type low3;
-    HighSet<R, SYM, HIGH_ROW, true> high;     // [wide][full] below
-    HighSet<R, SYM, HIGH_ROW, false> high_part;
+    HighSet<R, SYM, HIGH_ROW, true> high;
     HighSet<R, SYM, WROW, true> wide;
-    HighSet<R, SYM, WROW, false> wide_part;
+    typename std::conditional<FP64, HighSet<R, SYM, HIGH_ROW, false>, NoLowSet<R>>::type high_part;
+    Tails<R, SYM, FP64 ? Cx<R>::T : WROW + 1, Cx<R>::T - 1> tails;
     bool nb3_ok = false;  // the three-buffer kernels' shared memory fits the device
     cudaError_t init(size_t smem_optin) {
         const int big = (int)pass_smem<R>(true, MAX_TABLE - 1, 1, std::is_same<R, float>::value);
         std::vector<KPtr> ks;
         low.all(ks);
         high.all(ks);
-        high_part.all(ks);
         wide.all(ks);
-        wide_part.all(ks);
+        high_part.all(ks);
+        tails.all(ks);
         for (KPtr k : ks) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
             if (e != cudaSuccess) return e;
@@ -803,6 +887,10 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
                 return set_error(QAOA_ECUDA, "plan: high pass rows of %d bits", ps.row);
             a.row = ps.row;
             a.lo = ps.lo;
+            if (!Kernels::FP64 && ps.bits < T - ps.row) {  // no carried bits: longer rows
+                a.row = T - ps.bits;
+                a.lo = pl.state_bits - ps.bits;
+            }
             a.active = ((1u << ps.bits) - 1u) << (T - ps.bits);
         }
         const bool last = i + 1 == seq.size();
@@ -857,30 +945,36 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
             }
             if (lrc) return lrc;
         } else {
-            // rows of HIGH_ROW or WROW bits; FULL kernels when no bit of the group is a carried one
-            const bool wide = ps.row != HIGH_ROW, full = ps.bits == T - ps.row;
-            const HighSet<R, SYM, HIGH_ROW, true> &hn = pk->high;
-            const HighSet<R, SYM, HIGH_ROW, false> &hp = pk->high_part;
-            const HighSet<R, SYM, Kernels::WROW, true> &wn = pk->wide;
-            const HighSet<R, SYM, Kernels::WROW, false> &wp = pk->wide_part;
-            if (L.mode == MODE_INIT) {
-                fill_table<R>(tab, r, 0, sign);
-                auto k = wide ? (full ? wn.init[u1] : wp.init[u1]) : (full ? hn.init[u1] : hp.init[u1]);
-                launch_pdl(k, grid, block, smem_phase, stream, a, *tab);
-            } else if (L.mode == MODE_FUSED) {
-                fill_table<R>(tab, r, L.la + 1, sign);
-                auto k = wide ? (full ? wn.fused[u1][u2] : wp.fused[u1][u2])
-                              : (full ? hn.fused[u1][u2] : hp.fused[u1][u2]);
-                const size_t smem_fused = pass_smem<R>(true, r.m, 1, early_landing<R, false, MODE_FUSED, 1>());
-                launch_pdl(k, grid, block, smem_fused, stream, a, *tab);
-            } else if (L.mode == MODE_PLAIN) {
-                auto k = a.reduce ? (wide ? (full ? wn.plain_red[u1] : wp.plain_red[u1])
-                                          : (full ? hn.plain_red[u1] : hp.plain_red[u1]))
-                                  : (wide ? (full ? wn.plain[u1] : wp.plain[u1])
-                                          : (full ? hn.plain[u1] : hp.plain[u1]));
-                launch_pdl(k, grid, block, smem_plain, stream, a, none);
-            } else {
+            if (L.mode != MODE_INIT && L.mode != MODE_PLAIN && L.mode != MODE_FUSED)
                 return set_error(QAOA_ECUDA, "schedule: phase-at-load on a strided pass");
+            auto launch_high = [&](const auto &hs) {
+                if (L.mode == MODE_FUSED) {
+                    fill_table<R>(tab, r, L.la + 1, sign);
+                    const size_t smem_fused = pass_smem<R>(true, r.m, 1, early_landing<R, false, MODE_FUSED, 1, HIGH_ROW>());
+                    launch_pdl(hs.fused[u1][u2], grid, block, smem_fused, stream, a, *tab);
+                } else if (L.mode == MODE_PLAIN) {
+                    launch_pdl(a.reduce ? hs.plain_red[u1] : hs.plain[u1], grid, block, smem_plain, stream, a, none);
+                }
+            };
+            auto launch_any = [&](const auto &hs) {
+                if (L.mode == MODE_INIT) {
+                    fill_table<R>(tab, r, 0, sign);
+                    launch_pdl(hs.init[u1], grid, block, smem_phase, stream, a, *tab);
+                } else {
+                    launch_high(hs);
+                }
+            };
+            const bool full = a.active == (((1u << T) - 1u) & ~((1u << a.row) - 1u));
+            if (full && a.row == HIGH_ROW) {
+                launch_any(pk->high);
+            } else if (full && a.row == Kernels::WROW) {
+                launch_any(pk->wide);
+            } else if constexpr (Kernels::FP64) {
+                if (a.row != HIGH_ROW) return set_error(QAOA_ECUDA, "plan: high pass rows of %d bits", a.row);
+                launch_any(pk->high_part);
+            } else {
+                if (L.mode == MODE_INIT) return set_error(QAOA_ECUDA, "schedule: a partial group first");
+                pk->tails.with(a.row, launch_high);
             }
         }
         rc = profile_after(kind, stream);

@@ -398,14 +398,17 @@ __device__ __forceinline__ void issue_tile(const typename G::V *st, const uint8_
     constexpr int JE = J1 < 0 ? NCH : J1;
     const uint32_t tid = threadIdx.x;
     if (state) {
-        // chunk q = tid + PT j covers tile elements [EPC q, EPC q + EPC)
-        // the bits of EPC * NT * j lie above those of EPC * tid and above the row
-        // bits, so the offset is linear in j
+        // chunk q = tid + PT j covers tile elements [EPC q, EPC q + EPC); the bits of
+        // EPC * NT * j lie above those of EPC * tid, and above the row bits too
+        // (so that the offset is linear in j) unless the rows are longer than one step
         const uint32_t off0 = base + elem_offset32((uint32_t)EPC * tid, row, lo);
         const uint32_t step = elem_offset32((uint32_t)(EPC * NT), row, lo);
         char *dst = reinterpret_cast<char *>(buf) + 16 * tid;
 #pragma unroll
-        for (int j = J0; j < JE; ++j) cp_async16(dst + (size_t)16 * NT * j, st + (off0 + step * j));
+        for (int j = J0; j < JE; ++j) {
+            const uint32_t o = (1 << row) > EPC * NT ? elem_offset32((uint32_t)(EPC * NT * j), row, lo) : step * j;
+            cp_async16(dst + (size_t)16 * NT * j, st + (off0 + o));
+        }
     }
     if (cost) {
         const uint32_t off0 = base + elem_offset32(16u * tid, row, lo);
@@ -416,6 +419,15 @@ __device__ __forceinline__ void issue_tile(const typename G::V *st, const uint8_
             cp_async16(sc + 16 * q + (PADC ? 16 * (q >> G::RB) : 0), cs + (off0 + step * j));
         }
     }
+}
+
+// A float as a double, by integer operations (the conversion instruction runs on
+// the FP64 pipe): the exponent rebiased by 896, the mantissa moved up.  Zeros,
+// subnormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f);
+    if (((b >> 23) & 0xFFu) - 1u >= 254u) return (double)f;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
 // |v|^2 for each arithmetic (double-float: in FP64).

@@ -44,7 +44,14 @@ def test_evolution(arith, n, p):
         assert abs(ps - rps) <= ps_tol * rps and abs(nm - 1) <= (1e-6 if dtype == "c64" else 1e-10)
 
 
-@pytest.mark.parametrize("arith,n,small,large", [("c64", 14, 3, 80), ("c128", 13, 5, 100), ("df64", 16, 2, 12)])
+# the large batches' second group has 1 .. 8 qubits (tiles with rows of 2^12 down to
+# 2^5 amplitudes in complex64, 2^11 down to 2^4 in double-float)
+@pytest.mark.parametrize("arith,n,small,large", [("c64", 14, 3, 80), ("c64", 15, 1, 40), ("c64", 16, 1, 20),
+                                                 ("c64", 17, 1, 12), ("c64", 18, 1, 12), ("c64", 19, 1, 6),
+                                                 ("c64", 20, 1, 4), ("c128", 13, 5, 100), ("c128", 17, 1, 12),
+                                                 ("df64", 13, 1, 100), ("df64", 14, 1, 60), ("df64", 15, 1, 30),
+                                                 ("df64", 16, 2, 12), ("df64", 17, 1, 12), ("df64", 18, 1, 6),
+                                                 ("df64", 19, 1, 6), ("df64", 20, 1, 4)])
 def test_batch_sizes_on_both_sides(arith, n, small, large):
     """`large` instances do not fit at once and run as HBM passes: the same states
     up to rounding, instance by instance."""
