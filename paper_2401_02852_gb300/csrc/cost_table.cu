@@ -49,15 +49,17 @@ namespace qaoa {
 constexpr int CT_THREADS = 256;
 constexpr int CT_CHUNK = 1024;     // clause records staged in shared memory at a time
 constexpr int CT_PARAM_M = 1023;   // largest m passed as kernel parameters
+constexpr int CT_PARAM_S = 240;    // ... in 4 KiB of them (13 us of host time a call, 22 with 16 KiB and the stats' memset)
 constexpr size_t ENCODE_MIN_LITS = 1 << 15;  // batches encoded on the device
 constexpr int NPL_SMALL = 10;      // bit planes for m <= 1023
 constexpr int NPL_LARGE = 13;      // bit planes for m <= 8191
 static_assert(QAOA_MAX_M < (1 << NPL_LARGE), "counts must fit the planes");
 
+template <int CAP>
 struct CostParams {
     int n, m;
     int mirror;  // count the lower half, write both (full tables, n >= 6)
-    ClauseRec rec[CT_PARAM_M];
+    ClauseRec rec[CAP];
 };
 
 __device__ __forceinline__ void csa(uint32_t &h, uint32_t &l, uint32_t a, uint32_t b, uint32_t c) {
@@ -113,13 +115,13 @@ struct WordCounter {
     }
 };
 
-// Adds to c0, c1 the counts of words X0, X1 against the clause records in
+// Adds to c0 (and, with WPT = 2, c1) the counts of words X0 (and X1) against the clause records in
 // shared memory (m16 = record count rounded up to 16; the padding records are
 // all zero, which are never violated: t = 0 = hi_mask selects
 // all_false | all_true = 0).
-template <int NPL>
-__device__ __forceinline__ void count_words2(uint32_t X0, uint32_t X1, int m16, const uint4 *srec,
-                                             WordCounter<NPL> &c0, WordCounter<NPL> &c1) {
+template <int NPL, int WPT>
+__device__ __forceinline__ void count_words(uint32_t X0, uint32_t X1, int m16, const uint4 *srec,
+                                            WordCounter<NPL> &c0, WordCounter<NPL> &c1) {
     const uint32_t xh0 = X0 << 5, xh1 = X1 << 5;
     for (int i0 = 0; i0 < m16; i0 += 16) {
         uint32_t v0[16], v1[16];
@@ -128,10 +130,10 @@ __device__ __forceinline__ void count_words2(uint32_t X0, uint32_t X1, int m16, 
             const uint4 r4 = srec[i0 + j];
             const ClauseRec r{r4.x, r4.y, r4.z, r4.w};
             v0[j] = violation_word(xh0, r);
-            v1[j] = violation_word(xh1, r);
+            if (WPT == 2) v1[j] = violation_word(xh1, r);
         }
         c0.add16(v0);
-        c1.add16(v1);
+        if (WPT == 2) c1.add16(v1);
     }
 }
 
@@ -214,16 +216,25 @@ __device__ __forceinline__ void emit_word(int n, uint64_t X, const uint32_t plan
     }
 }
 
-constexpr int SUB_WORDS = 2 * CT_THREADS;  // words per block step
-constexpr int SUB_BITS = 14;                // log2(32 SUB_WORDS): variables >= 14 are constant over a step
+// A block step takes WPT words per thread, WPT * CT_THREADS = 256 or 512 words:
+// variables >= 13 or 14 (sub_bits) are constant over it.  Two words per thread
+// share each record load and each filter; one word per thread gives small tables
+// twice the blocks and half the chain of clauses each, so it is taken while the
+// blocks of two do not fill the device twice (tables one after the other, with
+// their launches: n = 21, m = 168 20.3 -> 14.6 us, n = 23, m = 184 21.9 -> 14.5).
+template <int WPT>
+constexpr int sub_bits() {
+    return WPT == 2 ? 14 : 13;
+}
 
 // Keeps the clauses of recs[0, m) (m <= CT_CHUNK; shared or global memory)
-// that can be violated somewhere in the words [base, base + SUB_WORDS),
-// reduced to variables 5..13, in alive[0, *count), zero-padded to a multiple
+// that can be violated somewhere in the step's words from base on, reduced to
+// variables 5 .. sub_bits - 1, in alive[0, *count), zero-padded to a multiple
 // of 16.  Called by all threads of the block.
+template <int WPT>
 __device__ __forceinline__ int filter_clauses(uint32_t base, int m, const uint4 *recs, uint4 *alive, int *count) {
-    constexpr uint32_t MID = (1u << SUB_BITS) - 32u;  // variables 5..13
-    const uint32_t xu = base << 5;                     // x bits >= 14 of the step (bits < 14 are zero)
+    constexpr uint32_t MID = (1u << sub_bits<WPT>()) - 32u;
+    const uint32_t xu = base << 5;  // the constant x bits of the step (the others are zero)
     if (threadIdx.x == 0) *count = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -252,14 +263,15 @@ __device__ __forceinline__ int filter_clauses(uint32_t base, int m, const uint4 
     return c16;
 }
 
-// One table: each block steps through SUB_WORDS consecutive words at a time;
-// thread t takes words base + t and base + CT_THREADS + t, so every clause
-// record loaded from shared memory serves 64 assignments.  recs holds the m
+// One table: each block steps through WPT * CT_THREADS consecutive words at a
+// time; thread t takes word base + t and, with WPT = 2, base + CT_THREADS + t.
+// stats may be null.  recs holds the m
 // records (shared memory when m <= CT_CHUNK, else global), taken CT_CHUNK at a
 // time.
-template <int NPL>
+template <int NPL, int WPT>
 __device__ __forceinline__ void cost_table_body(int n, int m, const uint4 *recs, uint4 *alive, int *acount,
                                                 uint8_t *cost, unsigned long long *stats, bool mirror) {
+    constexpr int SUB_WORDS = WPT * CT_THREADS;
     mirror = mirror && n >= 6;  // the lower half is then a whole number of words
     const uint64_t words = n >= 5 ? (1ull << (n - 5)) >> (mirror ? 1 : 0) : 1ull;  // words counted
     const uint64_t steps = (words + SUB_WORDS - 1) / SUB_WORDS;
@@ -271,18 +283,21 @@ __device__ __forceinline__ void cost_table_body(int n, int m, const uint4 *recs,
         WordCounter<NPL> c0, c1;
         for (int k0 = 0; k0 < m || k0 == 0; k0 += CT_CHUNK) {
             const int mc = m - k0 < CT_CHUNK ? m - k0 : CT_CHUNK;
-            const int c16 = filter_clauses(base, mc, recs + k0, alive, acount);
-            if (X0 < words) count_words2<NPL>((uint32_t)X0, (uint32_t)(X1 < words ? X1 : X0), c16, alive, c0, c1);
+            const int c16 = filter_clauses<WPT>(base, mc, recs + k0, alive, acount);
+            if (X0 < words) count_words<NPL, WPT>((uint32_t)X0, (uint32_t)(X1 < words ? X1 : X0), c16, alive, c0, c1);
             __syncthreads();  // the list is rebuilt for the next chunk or step
         }
         if (X0 < words) {
             uint32_t p0[NPL], p1[NPL];
             c0.planes(p0);
-            c1.planes(p1);
             emit_word<NPL>(n, X0, p0, cost, nsol, mx, mirror);
-            if (X1 < words) emit_word<NPL>(n, X1, p1, cost, nsol, mx, mirror);
+            if (WPT == 2 && X1 < words) {
+                c1.planes(p1);
+                emit_word<NPL>(n, X1, p1, cost, nsol, mx, mirror);
+            }
         }
     }
+    if (!stats) return;
     // warp then block reduction, one atomic pair per block
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -311,10 +326,11 @@ __device__ __forceinline__ void cost_table_body(int n, int m, const uint4 *recs,
 
 // One table, m <= CT_PARAM_M, the records passed as kernel parameters and
 // copied to shared memory once.
-__global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_constant__ CostParams prm, uint8_t *cost,
-                                                                unsigned long long *stats) {
-    __shared__ uint4 srec[CT_CHUNK];
-    __shared__ uint4 alive[CT_CHUNK];
+template <int CAP, int WPT>
+__global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_constant__ CostParams<CAP> prm,
+                                                                uint8_t *cost, unsigned long long *stats) {
+    __shared__ uint4 srec[CAP];
+    __shared__ uint4 alive[CAP + 16];
     __shared__ int acount;
     for (int i = threadIdx.x; i < prm.m; i += CT_THREADS) {
         const ClauseRec r = prm.rec[i];
@@ -322,7 +338,7 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_con
     }
     __syncthreads();
     pdl_wait();
-    cost_table_body<NPL_SMALL>(prm.n, prm.m, srec, alive, &acount, cost, stats, prm.mirror != 0);
+    cost_table_body<NPL_SMALL, WPT>(prm.n, prm.m, srec, alive, &acount, cost, stats, prm.mirror != 0);
 }
 
 // Batched tables.  With ns == nullptr every instance has n qubits and its table
@@ -331,7 +347,7 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_con
 // shared memory once; longer lists are read from global memory chunk by chunk.
 // `bad` (nullable): set when the encoder found an invalid literal; nothing is
 // written then.
-template <int NPL>
+template <int NPL, int WPT>
 __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, const int *ns, const uint64_t *offs,
                                                                       const ClauseRec *recs, const int *ms,
                                                                       int m_stride, uint8_t *costs,
@@ -357,7 +373,7 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, con
     }
     const int ni = ns ? ns[inst] : n;
     uint8_t *dst = ns ? costs + offs[inst] : costs + ((size_t)inst << n);
-    cost_table_body<NPL>(ni, m, src, alive, &acount, dst, stats + 2 * inst, mirror != 0);
+    cost_table_body<NPL, WPT>(ni, m, src, alive, &acount, dst, stats + 2 * inst, mirror != 0);
 }
 
 // Clause records of a batch, one clause per thread, from the literals in host
@@ -458,10 +474,13 @@ int encode_instance(const naesat_instance *inst, ClauseRec *out) {
     return QAOA_OK;
 }
 
-static int grid_for(uint64_t words, int batch) {
+// Blocks per table, and the words per thread (see sub_bits).
+static int grid_for(uint64_t words, int batch, int *wpt) {
     DeviceInfo di;
     if (device_info(&di)) return -1;
-    const uint64_t need = ((words + 1) / 2 + CT_THREADS - 1) / CT_THREADS;
+    const uint64_t two = (words + 2 * CT_THREADS - 1) / (2 * CT_THREADS);
+    *wpt = two * (uint64_t)batch >= 2 * (uint64_t)di.sms ? 2 : 1;
+    const uint64_t need = *wpt == 2 ? two : (words + CT_THREADS - 1) / CT_THREADS;
     uint64_t cap = (uint64_t)di.sms * 8 * 4;
     cap = cap / (uint64_t)batch + 1;
     return (int)(need < cap ? need : cap);
@@ -471,16 +490,38 @@ int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d
                             const int *d_m, int m_stride, uint8_t *d_costs, unsigned long long *d_stats,
                             cudaStream_t stream, bool mirror, const unsigned long long *d_bad) {
     const uint64_t words = n >= 5 ? (1ull << (n - 5)) >> (mirror && n >= 6 ? 1 : 0) : 1ull;
-    const int gx = grid_for(words, batch);
+    int wpt = 2;
+    const int gx = grid_for(words, batch, &wpt);
     if (gx < 0) return QAOA_ECUDA;
     const int mi = mirror ? 1 : 0;
+    auto launch = [&](auto kernel) {
+        launch_pdl(kernel, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m, m_stride, d_costs,
+                   d_stats, mi, d_bad);
+    };
     profile_before(K_COST_TABLE, stream);
     if (m_stride <= CT_PARAM_M)
-        launch_pdl(cost_table_batch_kernel<NPL_SMALL>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
-                   m_stride, d_costs, d_stats, mi, d_bad);
+        wpt == 2 ? launch(cost_table_batch_kernel<NPL_SMALL, 2>) : launch(cost_table_batch_kernel<NPL_SMALL, 1>);
     else
-        launch_pdl(cost_table_batch_kernel<NPL_LARGE>, dim3(gx, batch), dim3(CT_THREADS), 0, stream, n, d_ns, d_offs, d_recs, d_m,
-                   m_stride, d_costs, d_stats, mi, d_bad);
+        wpt == 2 ? launch(cost_table_batch_kernel<NPL_LARGE, 2>) : launch(cost_table_batch_kernel<NPL_LARGE, 1>);
+    return profile_after(K_COST_TABLE, stream);
+}
+
+// One table whose records travel as kernel parameters.
+template <int CAP>
+static int launch_params(const naesat_instance *inst, int n, bool half, uint8_t *d_cost, unsigned long long *d_stats,
+                         cudaStream_t stream) {
+    CostParams<CAP> prm;
+    prm.n = n;
+    prm.m = inst->m;
+    prm.mirror = (!half && n >= 6) ? 1 : 0;  // a full table: count its lower half
+    encode_instance(inst, prm.rec);
+    const uint64_t words = prm.n >= 5 ? (1ull << (prm.n - 5)) >> prm.mirror : 1ull;
+    int wpt = 2;
+    const int gx = grid_for(words, 1, &wpt);
+    if (gx < 0) return QAOA_ECUDA;
+    profile_before(K_COST_TABLE, stream);
+    launch_pdl(wpt == 2 ? cost_table_kernel<CAP, 2> : cost_table_kernel<CAP, 1>, dim3(gx), dim3(CT_THREADS), 0, stream,
+               prm, d_cost, d_stats);
     return profile_after(K_COST_TABLE, stream);
 }
 
@@ -501,18 +542,8 @@ int launch_cost_table_one(const naesat_instance *inst, uint8_t *d_cost, unsigned
         QAOA_CUDA_TRY(cudaMemcpyAsync(d_m, &inst->m, sizeof(int), cudaMemcpyHostToDevice, stream));
         return launch_cost_table_batch(1, n, nullptr, nullptr, d_rec, d_m, inst->m, d_cost, d_stats, stream, !half);
     }
-    std::vector<char> buf(sizeof(CostParams));
-    CostParams *prm = reinterpret_cast<CostParams *>(buf.data());
-    prm->n = n;
-    prm->m = inst->m;
-    prm->mirror = (!half && n >= 6) ? 1 : 0;  // a full table: count its lower half
-    encode_instance(inst, prm->rec);
-    const uint64_t words = prm->n >= 5 ? (1ull << (prm->n - 5)) >> prm->mirror : 1ull;
-    const int gx = grid_for(words, 1);
-    if (gx < 0) return QAOA_ECUDA;
-    profile_before(K_COST_TABLE, stream);
-    launch_pdl(cost_table_kernel, dim3(gx), dim3(CT_THREADS), 0, stream, *prm, d_cost, d_stats);
-    return profile_after(K_COST_TABLE, stream);
+    return inst->m <= CT_PARAM_S ? launch_params<CT_PARAM_S>(inst, n, half, d_cost, d_stats, stream)
+                                 : launch_params<CT_PARAM_M>(inst, n, half, d_cost, d_stats, stream);
 }
 
 size_t cost_table_big_bytes(int m) { return m > CT_PARAM_M ? (size_t)m * sizeof(ClauseRec) + 16 : 0; }
@@ -531,11 +562,14 @@ static int cost_table_common(const naesat_instance *inst, uint8_t *d_cost, uint6
     Scratch *sc = nullptr;
     rc = scratch_for(stream, 256 + cost_table_big_bytes(inst->m), 64, &sc);
     if (rc) return rc;
-    unsigned long long *d_stats = reinterpret_cast<unsigned long long *>(sc->dev);
-    QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, 2 * sizeof(unsigned long long), stream));
+    // the counts are needed for the results, and for the range check when a count
+    // may exceed the uint8 table
+    const bool want = n_sol || max_cost || inst->m > 255;
+    unsigned long long *d_stats = want ? reinterpret_cast<unsigned long long *>(sc->dev) : nullptr;
+    if (want) QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, 2 * sizeof(unsigned long long), stream));
     rc = launch_cost_table_one(inst, d_cost, d_stats, stream, half, reinterpret_cast<char *>(sc->dev) + 256);
     if (rc) return rc;
-    if (!n_sol && !max_cost && inst->m <= 255) return QAOA_OK;
+    if (!want) return QAOA_OK;
     unsigned long long *h = reinterpret_cast<unsigned long long *>(sc->host);
     QAOA_CUDA_TRY(cudaMemcpyAsync(h, d_stats, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
