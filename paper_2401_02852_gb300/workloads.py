@@ -127,7 +127,8 @@ def grad_workload(batch: int = 256, n: int = 22, p: int = 20, adam_steps: int = 
         _sync()
         t_grad = time.perf_counter() - t0
     # per-kind roofline: algorithmic bytes of each launch kind over its event time
-    es, N = 8, batch * (1 << n)
+    # (the tables are flip-symmetric, so every pass works on half of the amplitudes)
+    es, N = 8, batch * (1 << (n - 1))
     kinds = prof.stats
     roof = {}
     for kind, (count, ms) in kinds.items():
