@@ -230,7 +230,7 @@ constexpr int sub_bits() {
 // Keeps the clauses of recs[0, m) (m <= CT_CHUNK; shared or global memory)
 // that can be violated somewhere in the step's words from base on, reduced to
 // variables 5 .. sub_bits - 1, in alive[0, *count), zero-padded to a multiple
-// of 16.  Called by all threads of the block.
+// of 16, and alive[that count] all zero too.  Called by all threads of the block.
 template <int WPT>
 __device__ __forceinline__ int filter_clauses(uint32_t base, int m, const uint4 *recs, uint4 *alive, int *count) {
     constexpr uint32_t MID = (1u << sub_bits<WPT>()) - 32u;
@@ -258,19 +258,70 @@ __device__ __forceinline__ int filter_clauses(uint32_t base, int m, const uint4 
     }
     __syncthreads();
     const int c = *count, c16 = (c + 15) & ~15;
-    for (int i = c + threadIdx.x; i < c16; i += CT_THREADS) alive[i] = make_uint4(0, 0, 0, 0);
+    for (int i = c + threadIdx.x; i <= c16; i += CT_THREADS) alive[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     return c16;
 }
 
+// Long lists are filtered once more, by each warp for its own 32 WPT consecutive
+// words, over which three more variables are constant (x bits 11..13 or 10..12):
+// of a block's list of 9-literal clauses about 0.4 remain.  wl receives the
+// remaining clauses' places in alive, padded to a multiple of 16 with that of a
+// record that is never violated; the counts then read their records through it.
+// For short lists (under WARP_FILTER_MIN) the pass and the indirection cost what
+// they save.  256 x (n = 17, k = 9, about 3000 clauses): 545 -> 273 us; 128 x (n =
+// 19, k = 7, 830 clauses): 272 -> 181; 256 x (n = 15, k = 7, 660): 51 -> 38.
+constexpr int WARP_FILTER_MIN = 256;
+template <int WPT>
+__device__ __forceinline__ int warp_filter(uint32_t X, int c16, const uint4 *alive, uint16_t *wl) {
+    constexpr uint32_t MASK = WPT == 2 ? 7u << 11 : 7u << 10;
+    const uint32_t lane = threadIdx.x & 31, xw = X << 5;
+    int cnt = 0;
+    for (int i0 = 0; i0 < c16; i0 += 32) {
+        const int i = i0 + (int)lane;
+        const uint4 r = i < c16 ? alive[i] : make_uint4(0, 0, 0, 0);
+        const uint32_t um = r.x & MASK, tu = (xw ^ r.y) & um;
+        const bool keep = (r.z != 0u && tu == um) || (r.w != 0u && tu == 0u);
+        const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, keep);
+        if (keep) wl[cnt + __popc(ballot & ((1u << lane) - 1u))] = (uint16_t)i;
+        cnt += __popc(ballot);
+    }
+    const int w16 = (cnt + 15) & ~15;
+    if (cnt + (int)lane < w16) wl[cnt + lane] = (uint16_t)c16;
+    __syncwarp();
+    return w16;
+}
+
+// count_words over the listed records.
+template <int NPL, int WPT>
+__device__ __forceinline__ void count_listed(uint32_t X0, uint32_t X1, int w16, const uint4 *alive, const uint16_t *wl,
+                                             WordCounter<NPL> &c0, WordCounter<NPL> &c1) {
+    const uint32_t xh0 = X0 << 5, xh1 = X1 << 5;
+    for (int i0 = 0; i0 < w16; i0 += 16) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(wl + i0), b = *reinterpret_cast<const uint4 *>(wl + i0 + 8);
+        const uint32_t ix[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        uint32_t v0[16], v1[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const uint4 r4 = alive[(j & 1) ? ix[j / 2] >> 16 : ix[j / 2] & 0xFFFFu];
+            const ClauseRec r{r4.x, r4.y, r4.z, r4.w};
+            v0[j] = violation_word(xh0, r);
+            if (WPT == 2) v1[j] = violation_word(xh1, r);
+        }
+        c0.add16(v0);
+        if (WPT == 2) c1.add16(v1);
+    }
+}
+
 // One table: each block steps through WPT * CT_THREADS consecutive words at a
-// time; thread t takes word base + t and, with WPT = 2, base + CT_THREADS + t.
-// stats may be null.  recs holds the m
-// records (shared memory when m <= CT_CHUNK, else global), taken CT_CHUNK at a
-// time.
+// time; a warp takes 32 WPT consecutive ones, lane t of it the t-th and, with WPT
+// = 2, the (32 + t)-th.  wl: null, or CT_CHUNK places per warp for the second
+// filter.  stats may be null.  recs holds the m records (shared or global
+// memory), taken CT_CHUNK at a time.
 template <int NPL, int WPT>
 __device__ __forceinline__ void cost_table_body(int n, int m, const uint4 *recs, uint4 *alive, int *acount,
-                                                uint8_t *cost, unsigned long long *stats, bool mirror) {
+                                                uint8_t *cost, unsigned long long *stats, bool mirror,
+                                                uint16_t *wl) {
     constexpr int SUB_WORDS = WPT * CT_THREADS;
     mirror = mirror && n >= 6;  // the lower half is then a whole number of words
     const uint64_t words = n >= 5 ? (1ull << (n - 5)) >> (mirror ? 1 : 0) : 1ull;  // words counted
@@ -279,12 +330,20 @@ __device__ __forceinline__ void cost_table_body(int n, int m, const uint4 *recs,
     uint32_t mx = 0;
     for (uint64_t sb = blockIdx.x; sb < steps; sb += gridDim.x) {
         const uint32_t base = (uint32_t)(sb * SUB_WORDS);
-        const uint64_t X0 = base + threadIdx.x, X1 = X0 + CT_THREADS;
+        const uint32_t Xw = base + (threadIdx.x >> 5) * (32 * WPT);  // the warp's first word
+        const uint64_t X0 = Xw + (threadIdx.x & 31), X1 = X0 + 32;
         WordCounter<NPL> c0, c1;
         for (int k0 = 0; k0 < m || k0 == 0; k0 += CT_CHUNK) {
             const int mc = m - k0 < CT_CHUNK ? m - k0 : CT_CHUNK;
             const int c16 = filter_clauses<WPT>(base, mc, recs + k0, alive, acount);
-            if (X0 < words) count_words<NPL, WPT>((uint32_t)X0, (uint32_t)(X1 < words ? X1 : X0), c16, alive, c0, c1);
+            const uint32_t X1c = (uint32_t)(X1 < words ? X1 : X0);
+            if (wl && c16 >= WARP_FILTER_MIN) {
+                uint16_t *mine = wl + (threadIdx.x >> 5) * CT_CHUNK;
+                const int w16 = warp_filter<WPT>(Xw, c16, alive, mine);
+                if (X0 < words) count_listed<NPL, WPT>((uint32_t)X0, X1c, w16, alive, mine, c0, c1);
+            } else if (X0 < words) {
+                count_words<NPL, WPT>((uint32_t)X0, X1c, c16, alive, c0, c1);
+            }
             __syncthreads();  // the list is rebuilt for the next chunk or step
         }
         if (X0 < words) {
@@ -338,13 +397,13 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_kernel(const __grid_con
     }
     __syncthreads();
     pdl_wait();
-    cost_table_body<NPL_SMALL, WPT>(prm.n, prm.m, srec, alive, &acount, cost, stats, prm.mirror != 0);
+    cost_table_body<NPL_SMALL, WPT>(prm.n, prm.m, srec, alive, &acount, cost, stats, prm.mirror != 0, nullptr);
 }
 
 // Batched tables.  With ns == nullptr every instance has n qubits and its table
 // at costs + inst 2^n; otherwise instance inst has ns[inst] qubits and its table
-// at costs + offs[inst].  Records of up to CT_CHUNK clauses are copied to
-// shared memory once; longer lists are read from global memory chunk by chunk.
+// at costs + offs[inst].  The records are read from global memory (each once per
+// block step) CT_CHUNK at a time.
 // `bad` (nullable): set when the encoder found an invalid literal; nothing is
 // written then.
 template <int NPL, int WPT>
@@ -354,26 +413,17 @@ __global__ void __launch_bounds__(CT_THREADS) cost_table_batch_kernel(int n, con
                                                                       unsigned long long *stats, int mirror,
                                                                       const unsigned long long *bad) {
     static_assert(sizeof(ClauseRec) == sizeof(uint4), "a clause record is one 16-byte load");
-    __shared__ uint4 srec[CT_CHUNK];
-    __shared__ uint4 alive[CT_CHUNK];
+    __shared__ uint4 alive[CT_CHUNK + 16];
+    __shared__ __align__(16) uint16_t wl[(CT_THREADS / 32) * CT_CHUNK];
     __shared__ int acount;
     pdl_wait();
     if (bad && *bad) return;
     const int inst = blockIdx.y;
     const int m = ms[inst];
-    const ClauseRec *g = recs + (size_t)inst * m_stride;
-    const uint4 *src = reinterpret_cast<const uint4 *>(g);
-    if (m <= CT_CHUNK) {
-        for (int i = threadIdx.x; i < m; i += CT_THREADS) {
-            const ClauseRec r = g[i];
-            srec[i] = make_uint4(r.hi_mask, r.hi_neg, r.all_true, r.all_false);
-        }
-        __syncthreads();
-        src = srec;
-    }
+    const uint4 *src = reinterpret_cast<const uint4 *>(recs + (size_t)inst * m_stride);
     const int ni = ns ? ns[inst] : n;
     uint8_t *dst = ns ? costs + offs[inst] : costs + ((size_t)inst << n);
-    cost_table_body<NPL, WPT>(ni, m, src, alive, &acount, dst, stats + 2 * inst, mirror != 0);
+    cost_table_body<NPL, WPT>(ni, m, src, alive, &acount, dst, stats + 2 * inst, mirror != 0, wl);
 }
 
 // Clause records of a batch, one clause per thread, from the literals in host
