@@ -134,6 +134,13 @@ def algorithmic_bytes(n: int, p: int, dtype: str):
     return out
 
 
+def moved_bytes(alg: dict, n: int, dtype: str):
+    """Per-kind bytes of an evolution on a flip-symmetric table: half of the
+    schedule's, and the other half of the state written by the last (high) pass."""
+    es = 8 if dtype == "c64" else 16
+    return {"pass_low": alg["pass_low"] // 2, "pass_high": alg["pass_high"] // 2 + es * 2 ** (n - 1)}
+
+
 def profiled_traffic(kind: str, n: int, p: int, dtype: str):
     """DRAM bytes per launch of `kind` (dram__bytes_read.sum + dram__bytes_write.sum,
     averaged over one step's launches of that kind) from the committed ncu summary
@@ -197,7 +204,7 @@ def config2_seeds(n: int, p: int, g, b, count: int = 5) -> dict:
     gold = load_golden("n30_p10_oracle.json") or {"instances": []}
     by_index = {r["index"]: r for r in gold["instances"]}
     alg = algorithmic_bytes(n, p, "c64")
-    sched = alg["pass_low"] + alg["pass_high"]
+    sched = sum(moved_bytes(alg, n, "c64").values())
     cost = torch.empty(1 << n, dtype=torch.uint8, device="cuda")
     st = torch.empty(1 << n, dtype=torch.complex64, device="cuda")
     st128 = torch.empty(1 << n, dtype=torch.complex128, device="cuda")
@@ -428,7 +435,7 @@ def run_native(args, ws, rank, local):
     # the schedule's amplitudes and the last one writes the other half too.
     kinds = prof.stats
     alg = algorithmic_bytes(n, p, dtype)
-    moved = {"pass_low": alg["pass_low"] // 2, "pass_high": alg["pass_high"] // 2 + es * 2 ** (n - 1)}
+    moved = moved_bytes(alg, n, dtype)
     peak, peak_src = measured_peak()
     per_unit = 2 * es + 1
     units = (2 ** n) * p

@@ -129,7 +129,8 @@ int naesat_cost_table_half(const naesat_instance *inst, uint8_t *d_cost_half, ui
                            uint32_t *max_cost, void *stream);
 
 /* Same for `batch` instances of one n: d_costs is device uint8 [batch][2^n];
- * n_sol / max_cost are host arrays [batch] (nullable). */
+ * n_sol / max_cost are host arrays [batch] (nullable).  Large batches' clause
+ * arrays may be read by the device during the call (which synchronises). */
 int naesat_cost_table_batch(int batch, const naesat_instance *insts, uint8_t *d_costs,
                             uint64_t *n_sol, uint32_t *max_cost, void *stream);
 
@@ -147,6 +148,9 @@ int naesat_cost_table_batch(int batch, const naesat_instance *insts, uint8_t *d_
  *   p_succ, norm  host, nullable: p_succ = sum_{C(x)=0} |psi(x)|^2 (Def. of the
  *            success probability, unnormalised) and sum_x |psi(x)|^2, reduced
  *            in FP64 inside the last pass.
+ * A flip-symmetric table, C(x) = C(2^n - 1 - x) for every x, as every NAE table is
+ * (checked on the device), is evolved on the x with bit n-1 clear, the others
+ * written as their mirror; any other table on every x.
  * Synchronises the stream when p_succ or norm is requested. */
 int qaoa_evolve(int n, const uint8_t *d_cost, int m, int p, const double *gamma, const double *beta,
                 int dtype, int flags, void *d_state, double *p_succ, double *norm, void *stream);
@@ -273,8 +277,8 @@ typedef struct {
     int n_streams;           /* CUDA streams for large requests (0 = 4)                       */
     int dtype;               /* QAOA_C64 or QAOA_C128                                          */
     int small_n_max;         /* n at or below which requests are packed (0 = default)         */
-    int flags;               /* mixer sign flags as for qaoa_evolve; QAOA_Z2_HALF runs the
-                                unpacked requests on the halved state (half the memory);
+    int flags;               /* mixer sign flags as for qaoa_evolve; unpacked requests run on the
+                                halved state, and QAOA_Z2_HALF charges them half the bytes;
                                 QAOA_DF64 (QAOA_C128 without QAOA_Z2_HALF) runs every request
                                 in double-float arithmetic                                    */
     int device;              /* CUDA device ordinal                                            */
@@ -318,7 +322,10 @@ int qaoa_server_destroy(qaoa_server *s);
  * the high passes work on n - 1 index bits) is split into HBM passes.  Pass 0 streams contiguous tiles and mixes qubits
  * [0, row_bits[0]).  Pass i > 0 streams tiles of 2^row_bits[i] contiguous
  * amplitudes times 2^G rows strided by 2^group_lo[i] (G = tile bits -
- * row_bits[i]) and mixes the top group_bits[i] qubits of its group.  Returns
+ * row_bits[i]) and mixes the top group_bits[i] qubits of its group; a last group
+ * with group_bits[i] < G may take that much longer rows in place of the bits it
+ * does not mix.  (Flip-symmetric full tables take the halved plan, whose groups are
+ * one bit lower; up to n = 20 an evolution may be one launch.)  Returns
  * the number of passes per layer (>= 1) or an error; arrays hold up to 8. */
 int qaoa_plan(int n, int dtype, int flags, int *group_lo, int *group_bits, int *row_bits);
 

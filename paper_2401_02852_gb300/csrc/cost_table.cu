@@ -13,10 +13,10 @@
 //   V = (t == 0 ? all_false : 0) | (t == hi_mask ? all_true : 0),
 // i.e. all literals false, or all true.  The 32 per-x counts are kept as
 // bit planes by a carry-save (Harley-Seal) adder over chunks of 16 clauses,
-// then transposed to bytes with 8x8 bit-matrix transposes.  The clause records
-// sit in shared memory (one broadcast 16-byte load per clause) and each thread
-// counts two words per record load.  The number of
-// solutions (count 0) and the largest count come out of the same pass.
+// then transposed to bytes with 8x8 bit-matrix transposes.  The records that a
+// block counts sit in shared memory (one broadcast 16-byte load per clause) and
+// each thread counts two words per record load.  The number of solutions (count
+// 0) and the largest count come out of the same pass.
 //
 // Large clause counts.  The records are staged CT_CHUNK at a time: the block
 // filters and counts one chunk, then the next, accumulating into the same
@@ -30,13 +30,14 @@
 // words), so a full table is counted on its lower half only: each counted
 // word is written twice, the second time byte-reversed at word W - 1 - X.
 //
-// Clause filtering.  A block takes 512 consecutive words at a time, so the
-// variables >= 14 (SUB_BITS) are constant over them.  A clause whose literals
-// on those variables are neither all true nor all false is violated nowhere in
-// the block; the block first keeps only the others, each reduced to its
-// variables 5..13 and to the one or two patterns still possible (for random
-// 5-literal clauses over 30 variables about 40% survive), then counts against
-// that list.  Counts are sums of 0/1 terms, so the list order is immaterial.
+// Clause filtering.  A block takes 512 consecutive words at a time (256 for small
+// tables), so the variables >= 14 (13) are constant over them.  A clause whose
+// literals on those variables are neither all true nor all false is violated
+// nowhere in the block; the block first keeps only the others, each reduced to
+// its remaining variables and to the one or two patterns still possible (for
+// random 5-literal clauses over 30 variables about 40% survive), then counts
+// against that list (long lists: against each warp's part of it).  Counts are sums
+// of 0/1 terms, so the list order is immaterial.
 #include <cuda_runtime.h>
 
 #include <cstring>
