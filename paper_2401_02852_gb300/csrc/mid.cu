@@ -33,7 +33,6 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include "orbits.cuh"
 #include "pass_common.cuh"
@@ -347,10 +346,12 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     char *d = reinterpret_cast<char *>(sc->dev);
     int *failed = reinterpret_cast<int *>(sc->host);
     double *result = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->host) + 64);
-    // pageable: the copy returns once the data is staged, so the call stays asynchronous
-    std::vector<char> h(tab + cof);
-    small_fill_layers(r.dtype, r.flags, r.n, r.m, r.p, r.gamma, r.beta, h.data(), h.data() + tab);
-    QAOA_CUDA_TRY(cudaMemcpyAsync(d, h.data(), h.size(), cudaMemcpyHostToDevice, stream));
+    Upload *up = nullptr;
+    if ((rc = upload_buffer(sc, tab + cof, &up))) return rc;
+    char *h = reinterpret_cast<char *>(up->host);
+    small_fill_layers(r.dtype, r.flags, r.n, r.m, r.p, r.gamma, r.beta, h, h + tab);
+    QAOA_CUDA_TRY(cudaMemcpyAsync(d, h, tab + cof, cudaMemcpyHostToDevice, stream));
+    if ((rc = upload_sent(up, stream))) return rc;
     MidArgs<R> a;
     a.cost = r.cost;
     a.state = reinterpret_cast<V *>(r.state);

@@ -35,6 +35,16 @@ int device_info(DeviceInfo *out);
 // ---------------------------------------------------------------------------
 // Per-(device, stream) scratch owned by the library.  Grows on demand; the
 // pinned host block receives results of device reductions.
+// Pinned host memory that an asynchronous upload reads after the call that
+// filled it has returned.
+struct Upload {
+    void *host = nullptr;
+    size_t bytes = 0;
+    cudaEvent_t sent = nullptr;  // recorded behind the upload
+    bool pending = false;
+};
+constexpr unsigned UPLOADS = 8;  // uploads in flight per stream before a call waits for the oldest
+
 struct Scratch {
     void *dev = nullptr;   // device bytes
     size_t dev_bytes = 0;
@@ -42,11 +52,19 @@ struct Scratch {
     size_t host_bytes = 0;
     unsigned *bars = nullptr;  // grid-barrier words, left fit for the next launch by each
     size_t n_bars = 0;
+    Upload up[UPLOADS];
+    unsigned next_up = 0;
 };
 // Returns scratch for `stream` on the current device with at least the given
 // capacities (device, pinned host).  Not thread-safe per stream: one caller
 // thread per stream at a time, as for any CUDA stream.
 int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratch **out);
+// Pinned memory of at least `bytes` for one upload, free of earlier ones (waits
+// for the oldest when UPLOADS are in flight); upload_sent once its copy is
+// enqueued.  The runtime may read a pageable source after cudaMemcpyAsync returns,
+// where it does not stage it; this memory stays until the copy is done.
+int upload_buffer(Scratch *s, size_t bytes, Upload **out);
+int upload_sent(Upload *u, cudaStream_t stream);
 // The stream's barrier words (at least `count`; kernels leave them as found).
 int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out);
 // Kernel attributes (the dynamic shared-memory limit) belong to a device:

@@ -108,6 +108,34 @@ int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratc
     return QAOA_OK;
 }
 
+int upload_buffer(Scratch *s, size_t bytes, Upload **out) {
+    Upload &u = s->up[s->next_up++ % UPLOADS];
+    if (u.pending) {
+        QAOA_CUDA_TRY(cudaEventSynchronize(u.sent));
+        u.pending = false;
+    }
+    if (!u.sent) QAOA_CUDA_TRY(cudaEventCreateWithFlags(&u.sent, cudaEventDisableTiming));
+    if (u.bytes < bytes) {
+        if (u.host) cudaFreeHost(u.host);
+        u.host = nullptr;
+        u.bytes = 0;
+        const size_t want = bytes < 16384 ? 16384 : bytes + bytes / 4;
+        if (cudaMallocHost(&u.host, want) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(QAOA_ENOMEM, "upload: cudaMallocHost(%zu) failed", want);
+        }
+        u.bytes = want;
+    }
+    *out = &u;
+    return QAOA_OK;
+}
+
+int upload_sent(Upload *u, cudaStream_t stream) {
+    QAOA_CUDA_TRY(cudaEventRecord(u->sent, stream));
+    u->pending = true;
+    return QAOA_OK;
+}
+
 int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out) {
     if (s->n_bars < count) {
         QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
@@ -136,6 +164,10 @@ static int release_all_scratch() {
         if (kv.second.dev) cudaFree(kv.second.dev);
         if (kv.second.host) cudaFreeHost(kv.second.host);
         if (kv.second.bars) cudaFree(kv.second.bars);
+        for (Upload &u : kv.second.up) {
+            if (u.host) cudaFreeHost(u.host);
+            if (u.sent) cudaEventDestroy(u.sent);
+        }
     }
     g_scratch.clear();
     cudaSetDevice(cur);
