@@ -41,7 +41,6 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
-#include <vector>
 
 #include "qaoa_internal.cuh"
 
@@ -577,20 +576,18 @@ static int launch_params(const naesat_instance *inst, int n, bool half, uint8_t 
 }
 
 int launch_cost_table_one(const naesat_instance *inst, uint8_t *d_cost, unsigned long long *d_stats,
-                          cudaStream_t stream, bool half, void *d_big) {
+                          cudaStream_t stream, bool half, void *d_big, void *h_big) {
     // the kernel uses n only for the number of assignments: the half table is
     // the first 2^(n-1) of them (variable n - 1 is 0 there)
     const int n = half ? inst->n - 1 : inst->n;
     if (inst->m > CT_PARAM_M) {
-        // records in global memory: d_big holds the m records then the count
-        if (!d_big) return set_error(QAOA_EINVAL, "m=%d needs device space for the clause records", inst->m);
-        std::vector<ClauseRec> rec((size_t)inst->m);
-        encode_instance(inst, rec.data());
-        ClauseRec *d_rec = reinterpret_cast<ClauseRec *>(d_big);
+        // records in global memory: d_big holds the m records then the count, from h_big
+        if (!d_big || !h_big) return set_error(QAOA_EINVAL, "m=%d needs space for the clause records", inst->m);
+        ClauseRec *d_rec = reinterpret_cast<ClauseRec *>(d_big), *h_rec = reinterpret_cast<ClauseRec *>(h_big);
         int *d_m = reinterpret_cast<int *>(d_rec + inst->m);
-        // pageable sources: the copies return once the data is staged
-        QAOA_CUDA_TRY(cudaMemcpyAsync(d_rec, rec.data(), rec.size() * sizeof(ClauseRec), cudaMemcpyHostToDevice, stream));
-        QAOA_CUDA_TRY(cudaMemcpyAsync(d_m, &inst->m, sizeof(int), cudaMemcpyHostToDevice, stream));
+        encode_instance(inst, h_rec);
+        *reinterpret_cast<int *>(h_rec + inst->m) = inst->m;
+        QAOA_CUDA_TRY(cudaMemcpyAsync(d_rec, h_rec, cost_table_big_bytes(inst->m), cudaMemcpyHostToDevice, stream));
         return launch_cost_table_batch(1, n, nullptr, nullptr, d_rec, d_m, inst->m, d_cost, d_stats, stream, !half);
     }
     return inst->m <= CT_PARAM_S ? launch_params<CT_PARAM_S>(inst, n, half, d_cost, d_stats, stream)
@@ -611,14 +608,15 @@ static int cost_table_common(const naesat_instance *inst, uint8_t *d_cost, uint6
     if (half && inst->n < 6) return set_error(QAOA_ERANGE, "half table needs n >= 6 (n=%d)", inst->n);
     cudaStream_t stream = (cudaStream_t)stream_;
     Scratch *sc = nullptr;
-    rc = scratch_for(stream, 256 + cost_table_big_bytes(inst->m), 64, &sc);
+    rc = scratch_for(stream, 256 + cost_table_big_bytes(inst->m), 256 + cost_table_big_bytes(inst->m), &sc);
     if (rc) return rc;
     // the counts are needed for the results, and for the range check when a count
     // may exceed the uint8 table
     const bool want = n_sol || max_cost || inst->m > 255;
     unsigned long long *d_stats = want ? reinterpret_cast<unsigned long long *>(sc->dev) : nullptr;
     if (want) QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, 2 * sizeof(unsigned long long), stream));
-    rc = launch_cost_table_one(inst, d_cost, d_stats, stream, half, reinterpret_cast<char *>(sc->dev) + 256);
+    rc = launch_cost_table_one(inst, d_cost, d_stats, stream, half, reinterpret_cast<char *>(sc->dev) + 256,
+                               reinterpret_cast<char *>(sc->host) + 256);
     if (rc) return rc;
     if (!want) return QAOA_OK;
     unsigned long long *h = reinterpret_cast<unsigned long long *>(sc->host);

@@ -236,10 +236,11 @@ int launch_cost_table_batch(int batch, int n, const int *d_ns, const uint64_t *d
                             const int *d_m, int m_stride, uint8_t *d_costs, unsigned long long *d_stats,
                             cudaStream_t stream, bool mirror, const unsigned long long *d_bad = nullptr);
 // One table.  Up to 1023 clauses the records go as kernel parameters (no
-// staging); a longer list is copied to d_big (device, cost_table_big_bytes(m)
-// bytes, 16-byte aligned) and counted chunk by chunk.
+// staging); a longer list is copied from h_big (pinned, and left alone until the
+// copy is done) to d_big (device), cost_table_big_bytes(m) bytes each, 16-byte
+// aligned, and counted chunk by chunk.
 int launch_cost_table_one(const naesat_instance *inst, uint8_t *d_cost, unsigned long long *d_stats,
-                          cudaStream_t stream, bool half, void *d_big);
+                          cudaStream_t stream, bool half, void *d_big, void *h_big);
 size_t cost_table_big_bytes(int m);
 
 // Multi-pass evolution of `batch` states (device side only, no host sync).

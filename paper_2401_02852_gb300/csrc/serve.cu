@@ -178,7 +178,9 @@ static int launch_large(qaoa_server *sv, Slot &s, Req &q) {
     unsigned long long *d_stats = reinterpret_cast<unsigned long long *>(s.d_stage);
     double *d_res = reinterpret_cast<double *>(s.d_stage + 16);
     QAOA_CUDA_TRY(cudaMemsetAsync(d_stats, 0, 16, s.stream));
-    if ((rc = launch_cost_table_one(&inst, (uint8_t *)s.d_cost, d_stats, s.stream, true, s.d_stage + 256))) return rc;
+    if ((rc = launch_cost_table_one(&inst, (uint8_t *)s.d_cost, d_stats, s.stream, true, s.d_stage + 256,
+                                    s.h_stage + 256)))
+        return rc;
     const int gx = pass_grid_x(dtype, q.n - 1, 1);
     if (gx < 0) return QAOA_ECUDA;
     if (s.part_cap < (size_t)gx * 2) {
