@@ -26,6 +26,11 @@
  *  - Every entry point returns an int status (QAOA_OK = 0, QAOA_PENDING > 0,
  *    errors < 0); no exception crosses the ABI.  qaoa_last_error() gives a
  *    thread-local message for the last failing call of the calling thread.
+ *  - Up to n = 20 an evolution may run as one launch whose CTAs wait for one
+ *    another, each wait with a limit of about a second.  If one runs out, the call
+ *    returns QAOA_ECUDA when it waits for the results; otherwise the next call on
+ *    that stream does, once (qaoa_success_prob, its variant and the running times
+ *    also when it ran out while they waited), and the evolution's state is not valid.
  *  - Arguments are validated on the host before any device work; an invalid
  *    call changes no device memory.
  */

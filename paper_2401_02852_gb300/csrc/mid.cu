@@ -54,8 +54,8 @@ struct MidArgs {
     double *partials;                    // [batch][G][2]
     double *result;                      // nullable: [batch][2]
     int *slots;                          // [batch][G] verdicts of the flip-symmetry check
-    unsigned *bar;                       // [batch][2]: arrivals (zero between launches), phase
-    int *failed;                         // set when a wait ran out
+    unsigned *bar;                       // [batch][2]: arrivals, phase (uploaded as zeros)
+    int *failed;                         // the stream's fault word: set when a wait ran out
     int n, m, p, T;
     int G;     // CTAs per instance
     int kmax;  // most generators per round
@@ -63,7 +63,7 @@ struct MidArgs {
 };
 
 // All CTAs of an instance arrive; the last one resets the count and flips the
-// phase the others wait for (so the words are as found after every launch).
+// phase the others wait for.
 __device__ __forceinline__ void instance_barrier(unsigned *bar, unsigned G, bool &dead, int *failed) {
     __syncthreads();
     if (threadIdx.x == 0 && !dead) {
@@ -337,30 +337,32 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     if ((rc = mid_capacity<R>(T, di, &cap))) return rc;
     if ((int64_t)r.batch * G > cap) return QAOA_OK;
     const size_t tab = small_table_bytes(sizeof(V), r.p, r.m), cof = sizeof(SmallCoef<R>) * (size_t)r.p;
+    const size_t bar = (tab + cof + 15) & ~(size_t)15, sent = bar + 2 * sizeof(unsigned) * (size_t)r.batch;
     const size_t part = sizeof(double) * 2 * (size_t)r.batch * G, slot = sizeof(int) * (size_t)r.batch * G;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     Scratch *sc = nullptr;
-    if ((rc = scratch_for(stream, al(tab + cof) + al(part) + slot, 2 * sizeof(double) * (size_t)r.batch + 64, &sc))) return rc;
-    unsigned *bars = nullptr;
-    if ((rc = scratch_bars(stream, sc, 2 * (size_t)r.batch, &bars))) return rc;
+    if ((rc = scratch_for(stream, al(sent) + al(part) + slot, 2 * sizeof(double) * (size_t)r.batch, &sc))) return rc;
+    int *failed = nullptr;
+    if ((rc = fault_word(stream, &failed))) return rc;
     char *d = reinterpret_cast<char *>(sc->dev);
-    int *failed = reinterpret_cast<int *>(sc->host);
-    double *result = reinterpret_cast<double *>(reinterpret_cast<char *>(sc->host) + 64);
+    double *result = reinterpret_cast<double *>(sc->host);
+    // the tables, and the barrier words as zeros: whatever a launch before left
     Upload *up = nullptr;
-    if ((rc = upload_buffer(sc, tab + cof, &up))) return rc;
+    if ((rc = upload_buffer(sc, sent, &up))) return rc;
     char *h = reinterpret_cast<char *>(up->host);
     small_fill_layers(r.dtype, r.flags, r.n, r.m, r.p, r.gamma, r.beta, h, h + tab);
-    QAOA_CUDA_TRY(cudaMemcpyAsync(d, h, tab + cof, cudaMemcpyHostToDevice, stream));
+    memset(h + bar, 0, sent - bar);
+    QAOA_CUDA_TRY(cudaMemcpyAsync(d, h, sent, cudaMemcpyHostToDevice, stream));
     if ((rc = upload_sent(up, stream))) return rc;
     MidArgs<R> a;
     a.cost = r.cost;
     a.state = reinterpret_cast<V *>(r.state);
     a.tab = reinterpret_cast<const V *>(d);
     a.coef = reinterpret_cast<const SmallCoef<R> *>(d + tab);
-    a.partials = reinterpret_cast<double *>(d + al(tab + cof));
+    a.partials = reinterpret_cast<double *>(d + al(sent));
     a.result = h_result ? result : nullptr;
-    a.slots = reinterpret_cast<int *>(d + al(tab + cof) + al(part));
-    a.bar = bars;
+    a.slots = reinterpret_cast<int *>(d + al(sent) + al(part));
+    a.bar = reinterpret_cast<unsigned *>(d + bar);
     a.failed = failed;
     a.n = r.n;
     a.m = r.m;
@@ -371,7 +373,6 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     // then feed every quarter of the SM
     a.kmax = std::min(4, std::is_same<R, double>::value ? T - 7 : std::max(3, T - 7));
     a.half = (r.flags & QAOA_Z2_HALF) ? 1 : 0;
-    if (h_result) *failed = 0;
     void *args[] = {(void *)&a};
     profile_before(K_MID, stream);
     const cudaError_t e = cudaLaunchCooperativeKernel((const void *)mid_kernel<R>, dim3((unsigned)(r.batch * G)),
@@ -384,10 +385,7 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     *taken = true;
     if (!h_result) return QAOA_OK;
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
-    if (*failed) {
-        cudaMemsetAsync(bars, 0, 2 * sizeof(unsigned) * (size_t)r.batch, stream);
-        return set_error(QAOA_ECUDA, "a grid barrier of the evolution ran out of time");
-    }
+    if ((rc = stream_fault(stream))) return rc;
     memcpy(h_result, result, 2 * sizeof(double) * (size_t)r.batch);
     return QAOA_OK;
 }

@@ -1140,6 +1140,7 @@ extern "C" int qaoa_success_prob(int n, const uint8_t *d_cost, const void *d_sta
     double *h = reinterpret_cast<double *>(sc->host);
     QAOA_CUDA_TRY(cudaMemcpyAsync(h, d_res, 2 * sizeof(double), cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
+    if ((rc = stream_fault(stream))) return rc;  // the state may come from a launch that failed meanwhile
     *p_succ = h[0];
     *norm = h[1];
     return QAOA_OK;
@@ -1212,6 +1213,7 @@ extern "C" int qaoa_success_prob_noalloc(int n, const uint8_t *d_cost, const voi
     double h[2];  // pageable host copy: the runtime stages it, nothing is allocated here
     QAOA_CUDA_TRY(cudaMemcpyAsync(h, d_res, sizeof h, cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
+    if ((rc = stream_fault(stream))) return rc;  // the state may come from a launch that failed meanwhile
     *p_succ = h[0];
     *norm = h[1];
     return QAOA_OK;

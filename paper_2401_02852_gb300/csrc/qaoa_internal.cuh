@@ -50,8 +50,7 @@ struct Scratch {
     size_t dev_bytes = 0;
     void *host = nullptr;  // pinned host bytes
     size_t host_bytes = 0;
-    unsigned *bars = nullptr;  // grid-barrier words, left fit for the next launch by each
-    size_t n_bars = 0;
+    int *fault = nullptr;  // pinned: set by a kernel whose grid barrier ran out of time
     Upload up[UPLOADS];
     unsigned next_up = 0;
 };
@@ -65,8 +64,12 @@ int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratc
 // where it does not stage it; this memory stays until the copy is done.
 int upload_buffer(Scratch *s, size_t bytes, Upload **out);
 int upload_sent(Upload *u, cudaStream_t stream);
-// The stream's barrier words (at least `count`; kernels leave them as found).
-int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out);
+// The stream's fault word, kept apart from the blocks that calls reuse.  A kernel may
+// set it after its call has returned: scratch_for then refuses the next call on
+// the stream, and stream_fault reports it to a call that has waited for the
+// stream.  Reporting clears it.
+int fault_word(cudaStream_t stream, int **out);
+int stream_fault(cudaStream_t stream);
 // Kernel attributes (the dynamic shared-memory limit) belong to a device:
 // the current device's ordinal for per-device set-up state, or -1 with the
 // error recorded when it is out of [0, MAX_DEVICES).

@@ -74,11 +74,42 @@ int current_device_slot() {
     return dev;
 }
 
+// Reports and clears the fault word of a stream (lock held).
+static int report_fault(Scratch &s, cudaStream_t stream) {
+    if (!s.fault || !*static_cast<volatile int *>(s.fault)) return QAOA_OK;
+    cudaStreamSynchronize(stream);  // the launch that set it may still run
+    *s.fault = 0;
+    return set_error(QAOA_ECUDA, "a grid barrier of an evolution on this stream ran out of time: its state is not valid");
+}
+
+int stream_fault(cudaStream_t stream) {
+    int dev = 0;
+    QAOA_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    auto it = g_scratch.find({dev, stream});
+    return it == g_scratch.end() ? QAOA_OK : report_fault(it->second, stream);
+}
+
+int fault_word(cudaStream_t stream, int **out) {
+    int dev = 0;
+    QAOA_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(g_scratch_mu);
+    Scratch &s = g_scratch[{dev, stream}];
+    if (!s.fault) {
+        QAOA_CUDA_TRY(cudaMallocHost((void **)&s.fault, sizeof(int)));
+        *s.fault = 0;
+    }
+    *out = s.fault;
+    return QAOA_OK;
+}
+
 int scratch_for(cudaStream_t stream, size_t dev_bytes, size_t host_bytes, Scratch **out) {
     int dev = 0;
     QAOA_CUDA_TRY(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     Scratch &s = g_scratch[{dev, stream}];
+    const int rc = report_fault(s, stream);
+    if (rc) return rc;
     if (s.dev_bytes < dev_bytes) {
         // The stream may still use the old block: wait for it before freeing.
         QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
@@ -136,24 +167,6 @@ int upload_sent(Upload *u, cudaStream_t stream) {
     return QAOA_OK;
 }
 
-int scratch_bars(cudaStream_t stream, Scratch *s, size_t count, unsigned **out) {
-    if (s->n_bars < count) {
-        QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
-        if (s->bars) cudaFree(s->bars);
-        s->bars = nullptr;
-        s->n_bars = 0;
-        const size_t want = count < 1024 ? 1024 : count;
-        if (cudaMalloc((void **)&s->bars, want * sizeof(unsigned)) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(QAOA_ENOMEM, "scratch: %zu barrier words", want);
-        }
-        QAOA_CUDA_TRY(cudaMemsetAsync(s->bars, 0, want * sizeof(unsigned), stream));
-        s->n_bars = want;
-    }
-    *out = s->bars;
-    return QAOA_OK;
-}
-
 static int release_all_scratch() {
     std::lock_guard<std::mutex> lk(g_scratch_mu);
     int cur = 0;
@@ -163,7 +176,7 @@ static int release_all_scratch() {
         cudaDeviceSynchronize();
         if (kv.second.dev) cudaFree(kv.second.dev);
         if (kv.second.host) cudaFreeHost(kv.second.host);
-        if (kv.second.bars) cudaFree(kv.second.bars);
+        if (kv.second.fault) cudaFreeHost(kv.second.fault);
         for (Upload &u : kv.second.up) {
             if (u.host) cudaFreeHost(u.host);
             if (u.sent) cudaEventDestroy(u.sent);

@@ -480,6 +480,7 @@ static int sample_impl(int batch, int n, const uint8_t *d_costs, const void *d_s
     int *h = reinterpret_cast<int *>(sc->host);
     QAOA_CUDA_TRY(cudaMemcpyAsync(h, d_first, fb, cudaMemcpyDeviceToHost, stream));
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
+    if ((rc = stream_fault(stream))) return rc;  // the states may come from a launch that failed meanwhile
     for (int i = 0; i < batch; ++i) running_time[i] = h[i] >= k ? 0 : (int64_t)h[i] + 1;
     return QAOA_OK;
 }
