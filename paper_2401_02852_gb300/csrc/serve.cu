@@ -108,6 +108,9 @@ namespace qaoa {
 
 static size_t es_of(int dtype) { return dtype == QAOA_C64 ? 8 : 16; }
 
+// Bytes of a packed request's table: the next table's 16-byte stores start behind it.
+static size_t packed_table_bytes(int n) { return n < 4 ? 16 : (size_t)1 << n; }
+
 static int ensure_stage(Slot &s, size_t bytes) {
     if (s.stage_cap >= bytes) return QAOA_OK;
     if (s.h_stage) cudaFreeHost(s.h_stage);
@@ -272,7 +275,7 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
         max_n = std::max(max_n, q->n);
         tab_n += (size_t)std::max(q->p, 1) * (table_top(q->m) + 1);
         coef_n += (size_t)std::max(q->p, 1);
-        cost_bytes += ((size_t)1 << q->n);
+        cost_bytes += packed_table_bytes(q->n);
     }
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t o_recs = 0;
@@ -320,7 +323,7 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
         h_jobs[b] = j;
         toff += (size_t)pl * (mt + 1);
         coff += pl;
-        boff += (size_t)1 << q.n;
+        boff += packed_table_bytes(q.n);
     }
     QAOA_CUDA_TRY(cudaMemcpyAsync(d, h, o_up, cudaMemcpyHostToDevice, s.stream));
     QAOA_CUDA_TRY(cudaMemsetAsync(d + o_stats, 0, (size_t)B * 2 * sizeof(unsigned long long), s.stream));
@@ -344,7 +347,7 @@ static int launch_packed(qaoa_server *sv, Slot &s, std::vector<std::shared_ptr<R
 // and state, though the unpacked launches allocate half of each.
 static size_t footprint(const qaoa_server *sv, int n, bool packed) {
     const size_t N = (size_t)1 << n;
-    if (packed) return N;
+    if (packed) return packed_table_bytes(n);
     return ((sv->o.flags & QAOA_Z2_HALF) ? N / 2 : N) * (1 + es_of(sv->o.dtype));
 }
 
