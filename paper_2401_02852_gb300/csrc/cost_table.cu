@@ -644,16 +644,21 @@ extern "C" int naesat_cost_table_batch(int batch, const naesat_instance *insts, 
     const int n = insts[0].n;
     int m_stride = 1;
     size_t lits = 0;  // literals of the batch
+    bool aligned = true;
     for (int b = 0; b < batch; ++b) {
         int rc = valid_sizes(&insts[b]);
         if (rc) return rc;
         if (insts[b].n != n) return set_error(QAOA_EINVAL, "batch instances differ in n");
         m_stride = insts[b].m > m_stride ? insts[b].m : m_stride;
-        lits += insts[b].m > 0 ? (size_t)insts[b].m * insts[b].k : 0;
+        if (insts[b].m > 0) {
+            lits += (size_t)insts[b].m * insts[b].k;
+            aligned = aligned && (reinterpret_cast<uintptr_t>(insts[b].var) % sizeof(int32_t)) == 0;
+        }
     }
     // Short batches are checked and encoded here (about 3 ns a literal), without
-    // the encoder's launch and its first touch of the caller's memory.
-    const bool on_device = lits >= ENCODE_MIN_LITS && batch <= 65535;
+    // the encoder's launch and its first touch of the caller's memory; so are arrays at
+    // odd addresses (a record's field, say), which the host reads and the device cannot.
+    const bool on_device = lits >= ENCODE_MIN_LITS && batch <= 65535 && aligned;
     if (!on_device)
         for (int b = 0; b < batch; ++b) {
             int rc = validate_instance(&insts[b]);
