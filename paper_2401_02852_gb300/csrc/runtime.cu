@@ -27,6 +27,7 @@ int set_error(int code, const char *fmt, ...) {
 }
 
 int cuda_error(cudaError_t e, const char *what) {
+    cudaGetLastError();  // reported here: the next call's launch check must not find it again
     return set_error(QAOA_ECUDA, "%s: %s (%s)", what, cudaGetErrorString(e), cudaGetErrorName(e));
 }
 
