@@ -378,7 +378,10 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 2 
 // generators they sum to Im[conj(l00 + l11)(p01 + p10) + conj(l01 + l10)(p00 +
 // p11)], 12 operations instead of 16.  sigma^n and the phase are undone with the
 // forward table's conjugate, at the start of the next layer's first round
-// (local, like the cost bytes).  Two passes of FP64 work per layer and amplitude:
+// (local, like the cost bytes).  The powers of sigma and the sums of p_succ and the
+// norm are FP64 in complex64 too (32 x n = 12, p = 4, beta derivatives' error against
+// 80 bits 9.2e-8 with FP32 ones, 5.9e-8 with these; 100 x n = 12, p = 16 147 and 150
+// us).  Two passes of FP64 work per layer and amplitude:
 // 2 n + 4 operations forward, about 5.5 n + 11 backward.  (100 instances of n =
 // 12, p = 16 in FP64: 3.50 ms with one CTA per instance on the full states and
 // normalised radix-2 butterflies, 1.05 ms here; the operations alone take 0.83
@@ -468,14 +471,25 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
         const V *tab = stab + ((l + 1) & 1) * MAX_TABLE;
         const R A = cf.unit_a ? (R)1 : cf.A, B = cf.unit_a ? -cf.B : (R)-1;
         const bool ua = cf.unit_a != 0, seed = l == p - 1;
-        const R sg2 = (R)cf.sigma2;
+        const double sg2 = cf.sigma2, sg4 = sg2 * sg2;
+        // w after a round of K more generators (complex64: one multiplication in the chain)
+        auto weigh = [&](auto kc, double w) {
+            constexpr int K = decltype(kc)::value;
+            if constexpr (sizeof(R) == 4) {
+                return w * (K == 1 ? sg2 : (K == 2 ? sg4 : (K == 3 ? sg2 * sg4 : sg4 * sg4)));
+            } else {
+#pragma unroll
+                for (int q = 0; q < K; ++q) w *= sg2;
+                return w;
+            }
+        };
         if (!seed) ahead.fetch(tb + (size_t)l * (m + 1), m);
         if (l > 0) cf = cfs[l - 1];
-        R term = 0, w = 1;
-        double first0 = 0.0, first1 = 0.0;
+        double term = 0.0, w = 1.0;
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
             constexpr int K = decltype(kc)::value;
-            R t = 0, g0 = 0, g1 = 0;
+            R t = 0, g = 0;
+            double q0 = 0.0, q1 = 0.0;
             orbits<V, K>(pt.lb, j, mir, [&](const uint32_t(&off)[1 << K], uint32_t z0) {
                 V v[1 << K], u[1 << K];
 #pragma unroll
@@ -485,9 +499,14 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
 #pragma unroll
                     for (int r = 0; r < (1 << K); ++r) {
                         const bool sol = c[r] == 0;
-                        const R q = v[r].x * v[r].x + v[r].y * v[r].y;
-                        g1 += q;
-                        if (sol) g0 += q;
+                        double2 d;
+                        if constexpr (sizeof(R) == 4)
+                            d = make_double2(widen(v[r].x), widen(v[r].y));
+                        else
+                            d = amp_f64(v[r]);
+                        const double q = d.x * d.x + d.y * d.y;
+                        q1 += q;
+                        if (sol) q0 += q;
                         u[r].x = sol ? v[r].x : (R)0;
                         u[r].y = sol ? v[r].y : (R)0;
                     }
@@ -499,7 +518,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
 #pragma unroll
                         for (int r = 0; r < (1 << K); ++r) {
                             const int cst = min((int)c[r], m);
-                            g0 += (R)cst * (u[r].x * v[r].y - u[r].y * v[r].x);
+                            g += (R)cst * (u[r].x * v[r].y - u[r].y * v[r].x);
                             V ph = tab[cst];
                             ph.y = -ph.y;
                             v[r] = cmul(v[r], ph);
@@ -521,16 +540,13 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
                     at(sl, off[r]) = u[r];
                 }
             });
-            term = fma(w, t, term);
-#pragma unroll
-            for (int q = 0; q < K; ++q) w *= sg2;
+            term = fma(w, (double)t, term);
+            w = weigh(kc, w);
             if (first) {  // (p_succ, norm), or layer l + 1 done
-                first0 = (double)g0;
-                first1 = (double)g1;
                 if (seed)
-                    share(first0, first1);
+                    share(q0, q1);
                 else
-                    share(prev_term, prev_w * first0);
+                    share(prev_term, prev_w * (double)g);
             }
             if (last && !seed) ahead.put(stab + (l & 1) * MAX_TABLE);
             barrier<CB>(last);
@@ -563,13 +579,12 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
                     *where(sl, r) = u[r];
                 }
             });
-            term = fma(w, t, term);
-#pragma unroll
-            for (int q = 0; q < K; ++q) w *= sg2;
+            term = fma(w, (double)t, term);
+            w = weigh(kc, w);
             barrier<CB>(true);
         });
-        prev_term = (double)term;
-        prev_w = (double)w;
+        prev_term = term;
+        prev_w = w;
     }
     // layer 0's phase term
     R g = 0;
