@@ -400,10 +400,21 @@ LayerCoef layer_coef(double beta, int sign, int arith) {
 void phase_table(double gamma, double scale, int m, int arith, double *re, double *im) {
     if (arith != ARITH_F64) {
         constexpr int S = 8;
+        // exp(-i gamma k), the rounding of gamma k undone to first order (up to 2^26,
+        // where it is below 2^-27; beyond, the rounded angle stands)
+        auto turn = [gamma](double k, double *c, double *s) {
+            const double x = gamma * k, e = std::fabs(x) < 0x1p26 ? std::fma(gamma, k, -x) : 0.0;
+            const double cx = std::cos(x), sx = std::sin(x);
+            *c = cx - e * sx;
+            *s = -(sx + e * cx);
+        };
         double br[S], bi[S];
-        for (int b = 1; b < S; ++b) br[b] = std::cos(gamma * (double)b), bi[b] = -std::sin(gamma * (double)b);
+        for (int b = 1; b < S; ++b) turn((double)b, &br[b], &bi[b]);
         for (int c = 0; c <= m; c += S) {
-            const double x = scale * std::cos(gamma * (double)c), y = -scale * std::sin(gamma * (double)c);
+            double x, y;
+            turn((double)c, &x, &y);
+            x *= scale;
+            y *= scale;
             re[c] = x;
             im[c] = y;
             for (int b = 1; b < S && c + b <= m; ++b) {
