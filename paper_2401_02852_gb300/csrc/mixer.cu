@@ -199,12 +199,13 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
     };
     if (is_df<R>() && RED && reduce) {
         // The evolution's last pass: FP64 out, and the sums from the same values.
-        // Bound by the FP64 pipe, so the floats are widened by integer operations
-        // and only solutions add to p_succ: 5 FP64 operations per amplitude instead
-        // of about 11.
+        // Bound by the FP64 pipe, so the floats are widened by integer operations, and
+        // the solutions, which are few, are read back by the threads that hold one: 5
+        // FP64 operations per amplitude instead of about 11.  Their sum is compensated
+        // (Knuth's TwoSum), within an ulp or two whatever their number.
         double2 *sd = reinterpret_cast<double2 *>(sp);
         PairwiseSum<NR, double> nm;
-        double ps = 0.0;
+        uint32_t sols = 0;
         const uint32_t tid = threadIdx.x;
         const uint32_t cb = PADC ? cost_base<Cx<R>, LO>(tid) : 0u;
 #pragma unroll
@@ -213,12 +214,18 @@ __device__ __forceinline__ void store_tile(const typename Cx<R>::V *v, typename 
             const double2 d = make_double2(widen(w.x) + widen(w.y), widen(w.z) + widen(w.w));
             sd[off(r)] = d;
             if (mp) reinterpret_cast<double2 *>(mp)[-off(r)] = d;
-            const double pr = d.x * d.x + d.y * d.y;
-            nm.add(r, pr);
+            nm.add(r, d.x * d.x + d.y * d.y);
             const uint32_t u = tile_elem<Cx<R>, LO>(tid, r);
-            if (sc[PADC ? cb + Cx<R>::cidx((uint32_t)r << LO) : (Z2 ? land<Cx<R>::T>(u) : u)] == 0) ps += pr;
+            if (sc[PADC ? cb + Cx<R>::cidx((uint32_t)r << LO) : (Z2 ? land<Cx<R>::T>(u) : u)] == 0) sols |= 1u << r;
         }
-        acc[0] += ps;
+        double ps = 0.0, rest = 0.0;
+        for (; sols; sols &= sols - 1) {
+            const double2 d = sd[off(__ffs(sols) - 1)];  // this thread's own store
+            const double pr = d.x * d.x + d.y * d.y, s = ps + pr, back = s - ps;
+            rest += (ps - (s - back)) + (pr - back);
+            ps = s;
+        }
+        acc[0] += ps + rest;
         acc[1] += nm.total();
         return;
     } else if constexpr (is_df<R>()) {  // pairs renormalised between passes
