@@ -111,6 +111,22 @@ __device__ __forceinline__ long long weight(float2 z, int E) {
     return w.total();
 }
 
+
+// complex64 groups that hold an amplitude whose square is not finite in FP32 (their
+// exponent is stored plus ANY): one with a NaN or an infinity weighs 0, and E comes
+// from the others, their squares taken at 2^-130 where FP32 overflows; beside an
+// infinity E is at most -84, where ordinary amplitudes weigh 0 too.
+constexpr uint32_t INF_BITS = 0x7F800000u;
+constexpr int ANY = 4096;
+constexpr float DOWN = 2.710505431213761e-20f;  // 2^-65
+__device__ __forceinline__ bool finite(float2 z) {
+    return fabsf(z.x) < __uint_as_float(INF_BITS) && fabsf(z.y) < __uint_as_float(INF_BITS);
+}
+__device__ __forceinline__ void zero_nonfinite(float2 &z) {
+    if (!finite(z)) z = make_float2(0.f, 0.f);
+}
+__device__ __forceinline__ void zero_nonfinite(double2 &) {}  // no such groups
+
 __device__ __forceinline__ long long weight(double2 z, int E) {
     return scaled_trunc(z.x * z.x + z.y * z.y, E);
 }
@@ -125,7 +141,7 @@ __device__ __forceinline__ int scale_exp(float m) {
     return E < -200 ? -200 : (E > 200 ? 200 : E);
 }
 
-// Group g = blockIdx.x of instance blockIdx.y: E[g], the inclusive prefix Q
+// Group g = blockIdx.x of instance blockIdx.y: E[g] (or E[g] + ANY), the inclusive prefix Q
 // (int64) of its entries' weights, and the group total G[g] = Q_last 2^-E_g
 // in FP64.  With STAGED (complex64 states at 16-byte aligned addresses) the
 // group is first staged in shared memory (dynamic, STAGE_BYTES) with
@@ -178,35 +194,77 @@ __global__ void __launch_bounds__(GROUP, STAGED ? 3 : 1) entry_scan_kernel(const
     };
     __syncthreads();  // staged tile and smax
     long long wv = 0;
-    int E;
-    if (STAGED && ((uint64_t)(blockIdx.x + 1) << (GROUP_BITS + ENTRY_BITS)) <= N) {  // a whole group: entries in registers
+    int E, any = 0;
+    const bool whole = STAGED && ((uint64_t)(blockIdx.x + 1) << (GROUP_BITS + ENTRY_BITS)) <= N;
+    float4 w4[STAGED ? 16 : 1];  // a whole group: entries in registers
+    // the group's largest probability, as a float's bits: for complex64 infinities and
+    // NaN are above every finite one
+    unsigned mb = 0;
+    if (whole) {
         if constexpr (STAGED) {
-            float4 w[16];
-            float m = 0.f;
 #pragma unroll
             for (uint32_t j = 0; j < 16; ++j) {
-                w[j] = stage[16 * el + ((j + el) & 15u)];
-                m = fmaxf(m, fmaxf(prob_f(make_float2(w[j].x, w[j].y)), prob_f(make_float2(w[j].z, w[j].w))));
+                w4[j] = stage[16 * el + ((j + el) & 15u)];
+                mb = max(mb, max(__float_as_uint(prob_f(make_float2(w4[j].x, w4[j].y))),
+                                 __float_as_uint(prob_f(make_float2(w4[j].z, w4[j].w)))));
             }
-            const unsigned mb = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));  // nonnegative floats order as their bits
+            mb = __reduce_max_sync(0xFFFFFFFFu, mb);
             if ((el & 31u) == 0) atomicMax(&smax, mb);
+        }
+    } else {
+        if constexpr (sizeof(V) == 8) {
+            for (uint32_t i = 0; i < cnt; ++i) mb = max(mb, __float_as_uint(prob_f(amp(i))));
+        } else {
+            float m = 0.f;
+            for (uint32_t i = 0; i < cnt; ++i) m = fmaxf(m, prob_f(amp(i)));
+            mb = __float_as_uint(m);
+        }
+        atomicMax(&smax, mb);
+    }
+    __syncthreads();
+    E = scale_exp(__uint_as_float(smax));
+    if (sizeof(V) == 8 && smax >= INF_BITS) {
+        if constexpr (sizeof(V) == 8) {
+            __shared__ unsigned s_big;
             __syncthreads();
-            E = scale_exp(__uint_as_float(smax));
+            if (el == 0) smax = s_big = 0u;
+            __syncthreads();
+            float m = 0.f, big = 0.f;  // finite squares; those past FP32, down
+            int inf = 0;
+            for (uint32_t i = 0; i < cnt; ++i) {
+                const float2 z = amp(i);
+                const float pr = prob_f(z);
+                if (pr < __uint_as_float(INF_BITS))
+                    m = fmaxf(m, pr);
+                else if (finite(z))
+                    big = fmaxf(big, prob_f(make_float2(z.x * DOWN, z.y * DOWN)));
+                else if (pr == pr)
+                    inf = 1;
+            }
+            atomicMax(&smax, __float_as_uint(m));
+            atomicMax(&s_big, __float_as_uint(big));
+            inf = __syncthreads_or(inf);
+            E = s_big ? (W_TOP - ((int)(s_big >> 23) - 127 + 130)) & ~1 : scale_exp(__uint_as_float(smax));
+            if (inf) E = min(E, -84);
+            for (uint32_t i = 0; i < cnt; ++i) {
+                float2 z = amp(i);
+                zero_nonfinite(z);
+                wv += weight(z, E);
+            }
+            any = ANY;
+        }
+    } else if (whole) {
+        if constexpr (STAGED) {
             const float sc = pow2f(E / 2);
             WeightSum ws;
 #pragma unroll
             for (uint32_t j = 0; j < 16; ++j) {
-                ws.add(make_float2(w[j].x, w[j].y), sc);
-                ws.add(make_float2(w[j].z, w[j].w), sc);
+                ws.add(make_float2(w4[j].x, w4[j].y), sc);
+                ws.add(make_float2(w4[j].z, w4[j].w), sc);
             }
             wv = ws.total();
         }
     } else {
-        float m = 0.f;
-        for (uint32_t i = 0; i < cnt; ++i) m = fmaxf(m, prob_f(amp(i)));
-        atomicMax(&smax, __float_as_uint(m));
-        __syncthreads();
-        E = scale_exp(__uint_as_float(smax));
         for (uint32_t i = 0; i < cnt; ++i) wv += weight(amp(i), E);
     }
     // inclusive scan over the group's 256 entries (exact integer sums)
@@ -226,7 +284,7 @@ __global__ void __launch_bounds__(GROUP, STAGED ? 3 : 1) entry_scan_kernel(const
     const uint64_t gl = ne - ((uint64_t)blockIdx.x << GROUP_BITS);  // entries of this group
     if ((uint64_t)el == (gl < (uint64_t)GROUP ? gl : (uint64_t)GROUP) - 1) {
         G[inst * ng + blockIdx.x] = (double)incl * pow2d(-E);
-        Eg[inst * ng + blockIdx.x] = E;
+        Eg[inst * ng + blockIdx.x] = E + any;
     }
 }
 
@@ -357,7 +415,7 @@ __global__ void __launch_bounds__(DRAW_PT) draw_kernel(const V *states, int ns, 
     bool edge = ord(t) >= ord(total);
     auto dkey = [](double v) { return ord(v); };
     const uint64_t g = quad_search(Pi, (uint32_t)ng, ord(edge ? total : t), edge, dkey);
-    const int E = Eg[inst * ng + g];
+    const int Ea = Eg[inst * ng + g], any = sizeof(V) == 8 && Ea > ANY / 2 ? ANY : 0, E = Ea - any;
     // the remainder in the group's integer units
     const uint64_t e0 = g << GROUP_BITS;
     const uint64_t glen = ne - e0 < (uint64_t)GROUP ? ne - e0 : (uint64_t)GROUP;
@@ -375,6 +433,10 @@ __global__ void __launch_bounds__(DRAW_PT) draw_kernel(const V *states, int ns, 
     const uint64_t x0 = (e0 + e) << ENTRY_BITS;
     V z[8];
     load8(z, st, x0 + 8 * q, N, (reinterpret_cast<uintptr_t>(states) & 15u) == 0);
+    if (any) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) zero_nonfinite(z[i]);
+    }
     long long w[8], sum = 0;
     int last = -1;  // last amplitude of this lane with a weight
 #pragma unroll
