@@ -101,12 +101,12 @@ constexpr int TAB_REGS = MAX_TABLE / 128;  // at least 128 threads
 template <typename V>
 struct TabAhead {
     V e[TAB_REGS];
-    __device__ __forceinline__ void fetch(const V *tb, int m) {
+    __device__ __forceinline__ void fetch(const V *tb, int m, bool last = false) {
 #pragma unroll
         for (int k = 0; k < TAB_REGS; ++k) {
             const int c = (int)(threadIdx.x + k * blockDim.x);
             memset(&e[k], 0, sizeof(V));
-            if (c < MAX_TABLE && c <= m) e[k] = tb[c];
+            if (c < MAX_TABLE && (c <= m || last)) e[k] = tb[c <= m ? c : m];
         }
     }
     __device__ __forceinline__ void put(V *stab) const {

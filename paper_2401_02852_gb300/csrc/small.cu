@@ -205,14 +205,15 @@ __device__ __forceinline__ void load_costs(uint8_t *sc, const uint8_t *cost, uin
 }
 
 // p >= 1 layers forward from |+>; s holds the CTA's part afterwards.  tb0, cf0:
-// the layers' tables [p][m + 1] and coefficients [p].  On return the last
+// the layers' tables [p][m + 1] and coefficients [p].  LAST: a cost above m takes
+// the phase of m (gradients do, as their phase terms' weights).  On return the last
 // layer's table is in stab + ((p - 1) & 1) MAX_TABLE and the state is visible to
 // the whole cluster.
-template <typename R, int CB, typename V>
+template <typename R, int CB, bool LAST, typename V>
 __device__ __forceinline__ void forward_layers(const Part<V, CB> &pt, V *s, V *stab, const uint8_t *sc, int m, int p,
                                                const V *tb0, const SmallCoef<R> *cf0) {
     TabAhead<V> ahead;
-    ahead.fetch(tb0, m);
+    ahead.fetch(tb0, m, LAST);
     SmallCoef<R> cf = cf0[0];
     ahead.put(stab);
     __syncthreads();
@@ -221,7 +222,7 @@ __device__ __forceinline__ void forward_layers(const Part<V, CB> &pt, V *s, V *s
         const R A = cf.A, B = cf.B;
         const bool ua = cf.unit_a != 0, next = l + 1 < p;
         if (next) {
-            ahead.fetch(tb0 + (size_t)(l + 1) * (m + 1), m);
+            ahead.fetch(tb0 + (size_t)(l + 1) * (m + 1), m, LAST);
             cf = cf0[l + 1];
         }
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
@@ -315,7 +316,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 2 
                                    : reinterpret_cast<const SmallCoef<R> *>(
                                          prm.x + small_table_bytes(sizeof(V), max(jb.p, 1), jb.m));
     if (jb.p > 0) {
-        forward_layers<R, CB>(pt, s, stab, sc, jb.m, jb.p, tb, cf);
+        forward_layers<R, CB, false>(pt, s, stab, sc, jb.m, jb.p, tb, cf);
     } else {  // |+>: the table of "layer 0" holds the amplitude
         const V z = tb[0];
         for (uint32_t i = threadIdx.x; i < L; i += blockDim.x) s[i] = z;
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
     load_costs(sc, cost, pt.rank << pt.lb, L);
     const V *tb = reinterpret_cast<const V *>(tables);
     const SmallCoef<R> *cfs = reinterpret_cast<const SmallCoef<R> *>(coefs);
-    forward_layers<R, CB>(pt, s, stab, sc, m, p, tb, cfs);
+    forward_layers<R, CB, true>(pt, s, stab, sc, m, p, tb, cfs);
     double *o = out + (size_t)blockIdx.x * 2 * (1 + p);
     const double f = pt.sym ? 2.0 : 1.0;  // each amplitude stands for its complement too
     // The threads' shares of output row i, summed by the first warp: written
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
                 return w;
             }
         };
-        if (!seed) ahead.fetch(tb + (size_t)l * (m + 1), m);
+        if (!seed) ahead.fetch(tb + (size_t)l * (m + 1), m, true);
         if (l > 0) cf = cfs[l - 1];
         double term = 0.0, w = 1.0;
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
