@@ -40,9 +40,10 @@
 
 namespace qaoa {
 
-constexpr int MID_PT = 256;         // most threads per CTA
+constexpr int MID_PT = 128;         // threads per CTA
 constexpr int MID_ROW = 2;          // high tiles: rows of 4 amplitudes (32 or 64 bytes, whole sectors)
-constexpr int MID_T_MIN = 9, MID_T_MAX = 12;
+constexpr int MID_N_MAX = 20;       // largest n (see evolve_mid)
+constexpr int MID_T_MIN = 9, MID_T_MAX = (MID_N_MAX + MID_ROW + 1) / 2;
 constexpr unsigned MID_SPINS = 1u << 21;  // about a second of polls
 
 template <typename R>
@@ -109,7 +110,7 @@ __device__ __forceinline__ double2 stored(double2 v) { return v; }
 __device__ __forceinline__ float4 stored(float4 v) { return df_renorm(v); }
 
 template <typename R>
-__global__ void __launch_bounds__(MID_PT, 2) mid_kernel(const __grid_constant__ MidArgs<R> a) {
+__global__ void __launch_bounds__(MID_PT, 4) mid_kernel(const __grid_constant__ MidArgs<R> a) {
     using V = typename VecOf<R>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int T = a.T;
@@ -117,7 +118,8 @@ __global__ void __launch_bounds__(MID_PT, 2) mid_kernel(const __grid_constant__ 
     V *s = reinterpret_cast<V *>(smem_raw);
     V *stab = s + L;
     uint8_t *scs = reinterpret_cast<uint8_t *>(stab + MAX_TABLE);  // cost bytes of the low and of the high tile
-    const uint32_t G = (uint32_t)a.G, inst = blockIdx.x / G, c = blockIdx.x % G, nt = blockDim.x;
+    const uint32_t G = (uint32_t)a.G, inst = blockIdx.x / G, c = blockIdx.x % G;
+    constexpr uint32_t nt = MID_PT;
     const int sbits = a.half ? a.n - 1 : a.n;
     V *st = a.state + ((size_t)inst << sbits);
     const uint8_t *cost = a.cost + ((size_t)inst << sbits);
@@ -272,10 +274,7 @@ __global__ void __launch_bounds__(MID_PT, 2) mid_kernel(const __grid_constant__ 
         }
     }
     if (!a.result) return;
-    if (nt == MID_PT)
-        block_sum<2, MID_PT>(acc);
-    else
-        block_sum<2, 128>(acc);
+    block_sum<2, MID_PT>(acc);
     if (threadIdx.x == 0) {
         a.partials[2 * blockIdx.x] = acc[0];
         a.partials[2 * blockIdx.x + 1] = acc[1];
@@ -287,10 +286,7 @@ __global__ void __launch_bounds__(MID_PT, 2) mid_kernel(const __grid_constant__ 
         acc[0] += __ldcg(a.partials + 2 * (inst * G + i));
         acc[1] += __ldcg(a.partials + 2 * (inst * G + i) + 1);
     }
-    if (nt == MID_PT)
-        block_sum<2, MID_PT>(acc);
-    else
-        block_sum<2, 128>(acc);
+    block_sum<2, MID_PT>(acc);
     if (threadIdx.x == 0) {
         const double f = half && !a.half ? 2.0 : 1.0;  // the caller of a halved state doubles its results itself
         a.result[2 * inst] = f * acc[0];
@@ -298,15 +294,13 @@ __global__ void __launch_bounds__(MID_PT, 2) mid_kernel(const __grid_constant__ 
     }
 }
 
-// Tile bits for n qubits: two groups cover the state, T + (T - MID_ROW) >= n.
+// Tile bits for n qubits (at least 13): two groups cover the state, T + (T - MID_ROW) >= n.
 static int mid_tile(int n) { return std::max(MID_T_MIN, (n + MID_ROW + 1) / 2); }
 
 template <typename R>
 static size_t mid_smem(int T) {
     return sizeof(typename VecOf<R>::type) * ((size_t(1) << T) + MAX_TABLE) + 2 * (size_t(1) << T);
 }
-
-static int mid_threads(int T) { return T < MID_T_MAX ? 128 : MID_PT; }
 
 // CTAs of tile size T that the device holds at once.
 template <typename R>
@@ -320,7 +314,7 @@ static int mid_capacity(int T, const DeviceInfo &di, int *out) {
         QAOA_CUDA_TRY(cudaFuncSetAttribute(mid_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)mid_smem<R>(MID_T_MAX)));
         int per = 0;
-        QAOA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mid_kernel<R>, mid_threads(T), mid_smem<R>(T)));
+        QAOA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, mid_kernel<R>, MID_PT, mid_smem<R>(T)));
         cap[dev][T] = std::max(1, per * di.sms);
     }
     *out = cap[dev][T];
@@ -376,7 +370,7 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     void *args[] = {(void *)&a};
     profile_before(K_MID, stream);
     const cudaError_t e = cudaLaunchCooperativeKernel((const void *)mid_kernel<R>, dim3((unsigned)(r.batch * G)),
-                                                      dim3(mid_threads(T)), args, mid_smem<R>(T), stream);
+                                                      dim3(MID_PT), args, mid_smem<R>(T), stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {  // e.g. fewer SMs than the device's (a partition)
         cudaGetLastError();
         return QAOA_OK;
@@ -392,13 +386,11 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
 
 int evolve_mid(const EvolveReq &r, cudaStream_t stream, double *h_result, bool *taken) {
     *taken = false;
-    const int T = mid_tile(r.n);
-    if (r.p < 1 || T > MID_T_MAX || 2 * T < r.n + MID_ROW || r.n - 1 < T) return QAOA_OK;
     // Where the passes' tiles fill the device they are the better ones: n = 21, p =
     // 7 complex64 115 us against 138 here.  n = 20, p = 10: 157 / 148 us, in FP64
     // 1274 / 586, in double-float 372 / 286.  One complex64 layer is two passes
     // either way (n = 14: 49 / 53 us).
-    if (r.n > 20 || (r.dtype == QAOA_C64 && r.p < 2)) return QAOA_OK;
+    if (r.p < 1 || r.n > MID_N_MAX || (r.dtype == QAOA_C64 && r.p < 2)) return QAOA_OK;
     if ((reinterpret_cast<uintptr_t>(r.cost) | reinterpret_cast<uintptr_t>(r.state)) & 15u) return QAOA_OK;
     // a captured copy would read its host source again at every replay
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

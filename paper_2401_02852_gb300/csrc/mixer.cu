@@ -927,7 +927,7 @@ static int evolve_passes(const EvolveReq &r, double *d_partials, int gx, cudaStr
         const int u1 = a.ua1 ? 1 : 0, u2 = a.ua2 ? 1 : 0;
         const size_t smem_phase = pass_smem<R>(true, r.m), smem_plain = pass_smem<R>(false, 0);
         if (low) {
-            // the full-state or the halved-state set (double-float has only the former)
+            // the two- or the three-buffer set
             auto launch_low = [&](const auto &ls, dim3 g, size_t sm_phase, size_t sm_plain) -> int {
                 if (L.mode == MODE_INIT) {
                     fill_table<R>(tab, r, 0, sign);

@@ -330,24 +330,6 @@ __device__ __forceinline__ void mask_butterflies(typename G::V *v, uint32_t acti
     }
 }
 
-// Butterflies on the register bits of mapping LO whose tile bits are in `mask`
-// (bits LO + q, q = 0..RB-1) and below `below` (compile-time exclusion of bits
-// done in an earlier round).
-template <typename G, bool UA, int LO, int BELOW>
-__device__ __forceinline__ void reg_butterflies(typename G::V *v, uint32_t mask, typename G::Real A,
-                                                typename G::Real B) {
-    constexpr int RB = G::RB;
-    constexpr int NR = 1 << RB;
-#pragma unroll
-    for (int q = 0; q < RB; ++q) {
-        if (LO + q < BELOW && ((mask >> (LO + q)) & 1u)) {
-#pragma unroll
-            for (int i = 0; i < NR; ++i)
-                if (!(i & (1 << q))) bfly<UA>(v[i], v[i | (1 << q)], A, B);
-        }
-    }
-}
-
 // Re-distribute the tile from mapping FROM to mapping TO through shared memory
 // (padded layout: per-thread base + compile-time offset per register).  The
 // thread parts pass through an opaque asm so that the compiler recomputes them

@@ -603,9 +603,9 @@ int small_n_pack_limit(int dtype) { return dtype == QAOA_C64 ? 14 : 13; }
 
 // Dynamic shared memory of one CTA: `states` parts of the state (the whole one,
 // as an asymmetric table needs it), two phase tables, the cost bytes.
-static size_t small_smem(int dtype, int max_n, int cb, int states, int extra) {
+static size_t small_smem(int dtype, int max_n, int cb, int states) {
     const size_t es = dtype == QAOA_C64 ? sizeof(float2) : sizeof(double2), L = (size_t(1) << max_n) >> cb;
-    return es * (states * L + 2 * MAX_TABLE) + ((L + 15) & ~(size_t)15) + extra;
+    return es * (states * L + 2 * MAX_TABLE) + ((L + 15) & ~(size_t)15);
 }
 
 static int launch_clusters(const void *kernel, int n_clusters, int cb, int threads, size_t smem, cudaStream_t stream,
@@ -670,10 +670,10 @@ static int small_launch(int dtype, int flags, int count, const SmallJob *d_jobs,
                                 (const void *)small_kernel<double, 2>, (const void *)small_kernel<double, 3>};
     static const void *kf = (const void *)small_kernel<float, 0>, *kx = (const void *)small_kernel<dfloat, 0>;
     int rc = once_per_device(state, mu, [&] {
-        const int bf = (int)small_smem(QAOA_C64, small_n_pack_limit(QAOA_C64), 0, 1, 0);
+        const int bf = (int)small_smem(QAOA_C64, small_n_pack_limit(QAOA_C64), 0, 1);
         cudaError_t e = cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, bf);
         for (int c = 0; c < 4 && e == cudaSuccess; ++c) {
-            const int bd = (int)small_smem(QAOA_C128, small_n_pack_limit(QAOA_C128), c, 1, 0);
+            const int bd = (int)small_smem(QAOA_C128, small_n_pack_limit(QAOA_C128), c, 1);
             e = cudaFuncSetAttribute(kd[c], cudaFuncAttributeMaxDynamicSharedMemorySize, bd);
             if (c == 0 && e == cudaSuccess) e = cudaFuncSetAttribute(kx, cudaFuncAttributeMaxDynamicSharedMemorySize, bd);
         }
@@ -684,7 +684,7 @@ static int small_launch(int dtype, int flags, int count, const SmallJob *d_jobs,
     void *args[] = {(void *)&d_jobs, (void *)&all, (void *)&d_tables, (void *)&d_coefs, (void *)&max_n, (void *)&prm};
     const void *k = dtype == QAOA_C64 ? kf : ((flags & QAOA_DF64) ? kx : kd[cb]);
     profile_before(K_SMALL_N, stream);
-    rc = launch_clusters(k, count, cb, threads, small_smem(dtype, max_n, cb, 1, 0), stream, args);
+    rc = launch_clusters(k, count, cb, threads, small_smem(dtype, max_n, cb, 1), stream, args);
     if (rc) return rc;
     return profile_after(K_SMALL_N, stream);
 }
@@ -784,19 +784,21 @@ static int grad_small_impl(int batch, int n, const uint8_t *cost, int m, int p, 
                            int dtype, int flags, cudaStream_t stream, double *p_succ, double *dgamma, double *dbeta) {
     static std::mutex mu;
     static int state[MAX_DEVICES] = {};
-    static const void *ks[4] = {(const void *)small_grad_kernel<R, 0>, (const void *)small_grad_kernel<R, 1>,
-                                (const void *)small_grad_kernel<R, 2>, (const void *)small_grad_kernel<R, 3>};
+    constexpr int CBS = std::is_same<R, double>::value ? 3 : 0;  // clusters up to 2^CBS (small_cluster)
+    static const void *ks[4] = {(const void *)small_grad_kernel<R, 0>, (const void *)small_grad_kernel<R, CBS < 1 ? 0 : 1>,
+                                (const void *)small_grad_kernel<R, CBS < 2 ? 0 : 2>,
+                                (const void *)small_grad_kernel<R, CBS < 3 ? 0 : 3>};
     int rc = once_per_device(state, mu, [&] {
         cudaError_t e = cudaSuccess;
-        for (int c = 0; c < 4 && e == cudaSuccess; ++c)
+        for (int c = 0; c <= CBS && e == cudaSuccess; ++c)
             e = cudaFuncSetAttribute(ks[c], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)small_smem(dtype, small_n_limit(dtype), c, 2, 0));
+                                     (int)small_smem(dtype, small_n_limit(dtype), c, 2));
         return e;
     });
     if (rc) return rc;
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
-    const int cb = std::is_same<R, double>::value ? small_cluster(n, batch, di.sms) : 0;
+    const int cb = CBS > 0 ? small_cluster(n, batch, di.sms) : 0;
     const size_t tab = small_table_bytes(small_entry_bytes(dtype), p, m);
     const size_t in = (tab + small_coef_bytes(dtype) * (size_t)p + 255) & ~(size_t)255;
     Scratch *sc = nullptr;
@@ -809,7 +811,7 @@ static int grad_small_impl(int batch, int n, const uint8_t *cost, int m, int p, 
     const char *d_tab = d, *d_coef = d + tab;
     void *args[] = {(void *)&cost, (void *)&n, (void *)&m, (void *)&p, (void *)&d_tab, (void *)&d_coef, (void *)&h_out};
     profile_before(K_SMALL_N, stream);
-    rc = launch_clusters(ks[cb], batch, cb, cb == 0 ? SMALL_PT : SMALL_PT_CL, small_smem(dtype, n, cb, 2, 0), stream, args);
+    rc = launch_clusters(ks[cb], batch, cb, cb == 0 ? SMALL_PT : SMALL_PT_CL, small_smem(dtype, n, cb, 2), stream, args);
     if (rc) return rc;
     if ((rc = profile_after(K_SMALL_N, stream))) return rc;
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
