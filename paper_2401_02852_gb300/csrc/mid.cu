@@ -347,7 +347,9 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
     small_fill_layers(r.dtype, r.flags, r.n, r.m, r.p, r.gamma, r.beta, h, h + tab);
     memset(h + bar, 0, sent - bar);
     QAOA_CUDA_TRY(cudaMemcpyAsync(d, h, sent, cudaMemcpyHostToDevice, stream));
-    if ((rc = upload_sent(up, stream))) return rc;
+    // a call with results waits for the stream, its upload included (the event's record
+    // takes 3 to 4 us of such a call)
+    if (!h_result && (rc = upload_sent(up, stream))) return rc;
     MidArgs<R> a;
     a.cost = r.cost;
     a.state = reinterpret_cast<V *>(r.state);
@@ -373,9 +375,12 @@ static int mid_run(const EvolveReq &r, cudaStream_t stream, double *h_result, bo
                                                       dim3(MID_PT), args, mid_smem<R>(T), stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {  // e.g. fewer SMs than the device's (a partition)
         cudaGetLastError();
-        return QAOA_OK;
+        return h_result ? upload_sent(up, stream) : QAOA_OK;
     }
-    if ((rc = profile_after(K_MID, stream))) return rc;
+    if ((rc = profile_after(K_MID, stream))) {
+        if (h_result) cudaStreamSynchronize(stream);
+        return rc;
+    }
     *taken = true;
     if (!h_result) return QAOA_OK;
     QAOA_CUDA_TRY(cudaStreamSynchronize(stream));
