@@ -428,17 +428,17 @@ def run_native(args, ws, rank, local):
     # Roofline (the scored figure): the method's 1-pass floor, (2 es + 1) bytes per
     # amplitude-layer (17 B complex64, 33 B complex128: the state read and
     # written once and the cost byte read once per layer), times the
-    # amplitude-layers of a step, over the measured step time.  Extra passes of
-    # the schedule do not raise it.  Beside it, each pass kind's achieved
-    # bandwidth on the bytes it really moves (its launches' CUDA-event times):
-    # the table is flip-symmetric, C(x) = C(not x), so the passes work on half of
-    # the schedule's amplitudes and the last one writes the other half too.
+    # amplitude-layers that a step has to work on, over the measured step time.  The
+    # table is flip-symmetric, C(x) = C(not x), so those are half of the state's;
+    # extra passes of the schedule do not raise the figure.  Beside it, the bytes the
+    # passes really move (half of the schedule's, and the last one writes the other
+    # half too): over the step, and by pass kind over their CUDA-event times.
     kinds = prof.stats
     alg = algorithmic_bytes(n, p, dtype)
     moved = moved_bytes(alg, n, dtype)
     peak, peak_src = measured_peak()
     per_unit = 2 * es + 1
-    units = (2 ** n) * p
+    units = (2 ** (n - 1)) * p
     step_s = ms_max / args.steps / 1000.0
     achieved = per_unit * units / step_s / 1e9
     passes = {}
@@ -455,7 +455,8 @@ def run_native(args, ws, rank, local):
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
             "traffic_source": traffic_src, "peak_source": peak_src,
             "nominal_peak": NOMINAL_HBM_GBPS, "frac_of_nominal": achieved / NOMINAL_HBM_GBPS, "per_unit_bytes": per_unit,
-            "unit_name": "amplitude-layer", "units_per_step": units,
+            "unit_name": "amplitude-layer of the halved state", "units_per_step": units,
+            "moved_frac": (moved["pass_low"] + moved["pass_high"]) / step_s / 1e9 / peak,
             "achieved_pass_frac": passes[dom]["frac"] if dom else None, "dominant_pass_kind": dom,
             "passes": passes, "moved_bytes_per_step": moved["pass_low"] + moved["pass_high"],
             "schedule_bytes_per_step": alg["pass_low"] + alg["pass_high"]}

@@ -31,8 +31,9 @@
  *    returns QAOA_ECUDA when it waits for the results; otherwise the next call on
  *    that stream does, once (qaoa_success_prob, its variant and the running times
  *    also when it ran out while they waited), and the evolution's state is not valid.
- *  - Arguments are validated on the host before any device work; an invalid
- *    call changes no device memory.
+ *  - Arguments are validated before any result is written: on the host, except
+ *    that the literals of large batches of clauses are checked on the device.  An
+ *    invalid call changes none of the caller's memory.
  */
 #ifndef QAOA_NAESAT_H
 #define QAOA_NAESAT_H
@@ -156,6 +157,12 @@ int naesat_cost_table_batch(int batch, const naesat_instance *insts, uint8_t *d_
  * A flip-symmetric table, C(x) = C(2^n - 1 - x) for every x, as every NAE table is
  * (checked on the device), is evolved on the x with bit n-1 clear, the others
  * written as their mirror; any other table on every x.
+ * A call repeated with the same arguments gives the same bits.  The same instance
+ * alone, in a batch, in another batch's size or in a stream capture gives the same
+ * values up to rounding only: the kernel is chosen by n, p, the dtype and the batch
+ * (n <= 20: clusters while SMs are free, one launch while the batch fits the device
+ * at once and the stream is not capturing).  The server's results do not depend on
+ * what a request is packed or grouped with.
  * Synchronises the stream when p_succ or norm is requested. */
 int qaoa_evolve(int n, const uint8_t *d_cost, int m, int p, const double *gamma, const double *beta,
                 int dtype, int flags, void *d_state, double *p_succ, double *norm, void *stream);
