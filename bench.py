@@ -168,10 +168,10 @@ def profiled_traffic(kind: str, n: int, p: int, dtype: str):
 
 
 def step_traffic(n: int, p: int, dtype: str, alg: dict):
-    """DRAM bytes of one step (cost table + passes) from the committed per-kind
+    """DRAM bytes of one step (cost table, its symmetry check, passes) from the committed per-kind
     ncu figures, provided every kind the step launches has a current figure."""
     total, src = 0, None
-    launches = {"cost_table": 1, **alg["launches"]}
+    launches = {"cost_table": 1, "flip_check": 1, **alg["launches"]}
     for kind, count in launches.items():
         if not count:
             continue

@@ -254,10 +254,11 @@ def batch_workload(count: int = 100, n: int = 12, k: int = 3, r: float = 2.0, p:
         _, ps, nm = api.evolve_batch(n, costs, insts[0].m, g, b, "c128", out=states)
     _sync()
     dt = (time.perf_counter() - t0) / reps
-    # FP64 work of the whole-evolution kernel: per amplitude and layer, n factored
-    # butterfly stages (one FMA per component: 2 FMA per amplitude each) and the
-    # phase multiply (4 FMA-equivalents); 2 flops per FMA.
-    flops = count * (1 << n) * p * (2 * n + 4) * 2
+    # FP64 work of the whole-evolution kernel, on half of the amplitudes (the tables
+    # are flip-symmetric): per amplitude and layer, n factored butterfly stages (one
+    # FMA per component: 2 FMA per amplitude each) and the phase multiply (4
+    # FMA-equivalents); 2 flops per FMA.
+    flops = count * (1 << (n - 1)) * p * (2 * n + 4) * 2
     fp64_nominal = 1.25e12  # GB300 dense FP64, nominal (not measured here)
     # the same batch in double-float arithmetic (QAOA_DF64)
     from ._lib import DF64
