@@ -416,11 +416,11 @@ static int grad_passes(int batch, int n, const uint8_t *cost, int m, int p, cons
     if (rc) return rc;
     const int sign = (flags & QAOA_MIXER_RX2B) ? -1 : 1;
     // forward with the adjoint seed lam_p = P psi_p written by the last pass
-    const int gxf = pass_grid_x(dtype, n - 1, batch);
+    const int gxf = pass_grid_x(dtype, n, batch, true);
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
     const uint64_t tiles = 1ull << (n - AGeo<R>::T);
-    const int gxa = balanced_grid_x(di.sms * (sizeof(R) == 4 ? 2 : 1), batch, tiles / 2);
+    const int gxa = checked_grid_x(di.sms, di.sms * (sizeof(R) == 4 ? 2 : 1), batch, tiles);
     double *d_fpart = d_scr;                                  // batch * gxf * 2
     double *d_fres = d_fpart + (size_t)batch * gxf * 2;       // batch * 2
     double *d_apart = d_fres + (size_t)batch * 2;             // batch * p * gxa * 2
@@ -541,7 +541,7 @@ static int grad_common(int batch, int n, const uint8_t *cost, int m, int p, cons
         return grad_small(batch, n, cost, m, p, gamma, beta, dtype, flags, stream, p_succ, dgamma, dbeta);
     DeviceInfo di;
     if ((rc = device_info(&di))) return rc;
-    const int gxf = pass_grid_x(dtype, n - 1, batch);
+    const int gxf = pass_grid_x(dtype, n, batch, true);
     const size_t gxa = (size_t)di.sms * 2 + 1;
     const size_t words = (size_t)batch * gxf * 2 + (size_t)batch * 2 + (size_t)batch * p * gxa * 2 +
                          (size_t)batch * p * 2 + ((size_t)batch * flip_slots(n, batch, di.sms) + 1) / 2 + 64;
