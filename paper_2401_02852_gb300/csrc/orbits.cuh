@@ -15,12 +15,13 @@
 
 namespace qaoa {
 
-// One layer's coefficients, 32 bytes in complex128 and double-float.
+// One layer's coefficients, 32 bytes in complex128 and double-float.  sigma^2 is FP64,
+// or a double-float pair for complex64.
 template <typename R>
 struct SmallCoef {
     R A, B;
     int unit_a;
-    double sigma2;
+    typename std::conditional<sizeof(R) == 4, dfloat, double>::type sigma2;
 };
 static_assert(sizeof(SmallCoef<double>) == 32 && sizeof(SmallCoef<dfloat>) == 32, "one stride for complex128");
 

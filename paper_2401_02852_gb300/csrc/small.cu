@@ -379,10 +379,10 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 2 
 // generators they sum to Im[conj(l00 + l11)(p01 + p10) + conj(l01 + l10)(p00 +
 // p11)], 12 operations instead of 16.  sigma^n and the phase are undone with the
 // forward table's conjugate, at the start of the next layer's first round
-// (local, like the cost bytes).  The powers of sigma and the sums of p_succ and the
-// norm are FP64 in complex64 too (32 x n = 12, p = 4, beta derivatives' error against
-// 80 bits 9.2e-8 with FP32 ones, 5.9e-8 with these; 100 x n = 12, p = 16 147 and 150
-// us).  Two passes of FP64 work per layer and amplitude:
+// (local, like the cost bytes).  In complex64 the sums of p_succ and the norm are FP64
+// and the powers of sigma double-float products (32 x n = 12, p = 4, beta derivatives'
+// error against 80 bits 9.2e-8 with FP32 ones, 6.2e-8 with these; 100 x n = 12, p = 16 147
+// and 143 us).  Two passes of FP64 work per layer and amplitude:
 // 2 n + 4 operations forward, about 5.5 n + 11 backward.  (100 instances of n =
 // 12, p = 16 in FP64: 3.50 ms with one CTA per instance on the full states and
 // normalised radix-2 butterflies, 1.05 ms here; the operations alone take 0.83
@@ -416,6 +416,25 @@ __device__ __forceinline__ R pair_terms(const V *p, const V *l, R t) {
         }
     }
     return t;
+}
+
+// The weight sigma^(2 g) of a round after g generators, w sigma^(2 K) after the next: in
+// complex64 a double-float product, of which a round takes the nearest float.
+__device__ __forceinline__ double one_weight(double) { return 1.0; }
+__device__ __forceinline__ dfloat one_weight(dfloat) { return dfloat{1.f, 0.f}; }
+__device__ __forceinline__ double weight_of(double w) { return w; }
+__device__ __forceinline__ float weight_of(dfloat w) { return w.hi; }
+template <int K>
+__device__ __forceinline__ double weigh(double w, double s2) {
+#pragma unroll
+    for (int q = 0; q < K; ++q) w *= s2;
+    return w;
+}
+template <int K>
+__device__ __forceinline__ dfloat weigh(dfloat w, dfloat s2) {
+#pragma unroll
+    for (int q = 0; q < K; ++q) w = df_mul(w, s2.hi, s2.lo);
+    return w;
 }
 
 // out: [instance][CTA of its cluster][1 + p][2]: the CTA's share of (p_succ,
@@ -472,21 +491,11 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
         const V *tab = stab + ((l + 1) & 1) * MAX_TABLE;
         const R A = cf.unit_a ? (R)1 : cf.A, B = cf.unit_a ? -cf.B : (R)-1;
         const bool ua = cf.unit_a != 0, seed = l == p - 1;
-        const double sg2 = cf.sigma2, sg4 = sg2 * sg2;
-        // w after a round of K more generators (complex64: one multiplication in the chain)
-        auto weigh = [&](auto kc, double w) {
-            constexpr int K = decltype(kc)::value;
-            if constexpr (sizeof(R) == 4) {
-                return w * (K == 1 ? sg2 : (K == 2 ? sg4 : (K == 3 ? sg2 * sg4 : sg4 * sg4)));
-            } else {
-#pragma unroll
-                for (int q = 0; q < K; ++q) w *= sg2;
-                return w;
-            }
-        };
+        const auto sg2 = cf.sigma2;
         if (!seed) ahead.fetch(tb + (size_t)l * (m + 1), m, true);
         if (l > 0) cf = cfs[l - 1];
-        double term = 0.0, w = 1.0;
+        R term = 0;
+        auto w = one_weight(sg2);
         local_rounds(pt, [&](auto kc, int j, bool mir, bool first, bool last) {
             constexpr int K = decltype(kc)::value;
             R t = 0, g = 0;
@@ -541,8 +550,8 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
                     at(sl, off[r]) = u[r];
                 }
             });
-            term = fma(w, (double)t, term);
-            w = weigh(kc, w);
+            term = fma(weight_of(w), t, term);
+            w = weigh<K>(w, sg2);
             if (first) {  // (p_succ, norm), or layer l + 1 done
                 if (seed)
                     share(q0, q1);
@@ -580,12 +589,12 @@ __global__ void __launch_bounds__(CB == 0 ? SMALL_PT : SMALL_PT_CL, CB == 0 ? 1 
                     *where(sl, r) = u[r];
                 }
             });
-            term = fma(w, (double)t, term);
-            w = weigh(kc, w);
+            term = fma(weight_of(w), t, term);
+            w = weigh<K>(w, sg2);
             barrier<CB>(true);
         });
-        prev_term = term;
-        prev_w = w;
+        prev_term = (double)term;
+        prev_w = (double)weight_of(w);
     }
     // layer 0's phase term
     R g = 0;
@@ -717,7 +726,11 @@ static void fill_layer(int n, int m, double gamma, double beta, bool layer, bool
     }
     SmallCoef<R> *q = reinterpret_cast<SmallCoef<R> *>(coef);
     q->unit_a = k.unit_a ? 1 : 0;
-    q->sigma2 = layer_sigma2(k);
+    const double s2 = layer_sigma2(k);
+    if constexpr (sizeof(R) == 4)
+        q->sigma2 = dfloat{(float)s2, (float)(s2 - (double)(float)s2)};
+    else
+        q->sigma2 = s2;
     if constexpr (std::is_same<R, dfloat>::value) {
         const float a = (float)k.A, b = (float)k.B;
         q->A = dfloat{a, (float)(k.A - (double)a)};
