@@ -43,7 +43,7 @@ struct Upload {
     cudaEvent_t sent = nullptr;  // recorded behind the upload
     bool pending = false;
 };
-constexpr unsigned UPLOADS = 8;  // uploads in flight per stream before a call waits for the oldest
+constexpr unsigned UPLOADS = 32;  // uploads in flight per stream before a call waits for the oldest
 
 struct Scratch {
     void *dev = nullptr;   // device bytes
